@@ -1,99 +1,196 @@
-// Plain FP64 particle step (the reference GPU path): drift, TSC gather,
+// FP64 particle step (the reference GPU path): drift, TSC gather,
 // E-parallel cleaning, relativistic Boris kick-rotate-kick, drift, corrector
 // deposit at x^(n+1/2) and moments deposit at x^(n+1) (App. A.1-A.3 of
-// arXiv:1412.1087), in the oracle's arithmetic order.
+// arXiv:1412.1087), the particle arithmetic in double and in the oracle's
+// order but for the reciprocals.
 //
 // Same work decomposition as the mixed kernel (k_push_mixed.cu): persistent
 // CTAs take brick items from an atomic counter, stage the brick's fields plus
 // a halo in shared memory and accumulate the deposits in a shared int64
 // fixed-point tile that is added to the global accumulators at the end; a
 // particle whose stencil leaves the tile uses global memory directly.
+//
+// The FP64 pipe bounds it, so what need not be FP64 is not: the deposits are
+// integer products (wide_fixed.cuh), gamma and 1/gamma come from one
+// reciprocal square root (math64.cuh) instead of square roots and divisions,
+// positions are compared and cut into cell and offset with integer
+// operations: at 48^3 x 16 particles 4.40 -> 2.43 ms a push (1100 -> 440 FP64
+// operations a particle; the FP64 pipe is now 54% busy, and the shared 64-bit
+// atomics, compare-and-swap loops, are the longest waits).
+#include "math64.cuh"
 #include "push_common.cuh"
+#include "wide_fixed.cuh"
 
 namespace mhdpic {
 
 namespace {
 
+// Extra bits of a deposited quantity: |q| scale <= 2^62 / (9 * 64) (the
+// headroom of the scales), and up to 4 times that before the overflow flag,
+// so q 2^WIDE stays inside int64.
+constexpr int WIDE = 8;
+
 struct F64Const {
-    double dt, h, C, m, qn;
-    double scale[NCH];
-    double vlim[NCH];
+    double dt, h, C, C2, invC;
+    double lo[3], L[3], hi[3];   // box bounds
+    double inv_dx[3];
+    double mq[4];                // -m_CR times the corrector scales
+    double qn;                   // (q/mc) m / dV at the density's scale, and at the current's:
+    double qj[3];
+    uint64_t vlim[4];            // bits of the corrector quantities that raise the overflow flag
 };
 
+__device__ __forceinline__ void f64_const(const BoxDev &b, double dt, F64Const &k)
+{
+    k.dt = dt;
+    k.h = b.qm_cr * dt;
+    k.C = b.C;
+    k.C2 = b.C * b.C;
+    k.invC = 1.0 / b.C;
+    for (int d = 0; d < 3; ++d) {
+        k.lo[d] = b.x0[d];
+        k.L[d] = b.n[d] * b.dx[d];
+        k.hi[d] = k.lo[d] + k.L[d];
+        k.inv_dx[d] = b.inv_dx[d];
+    }
+    const double qn = b.qm_cr * b.m_cr * b.inv_dV;
+    k.qn = qn * b.scale[CH_N];
+    for (int d = 0; d < 3; ++d)
+        k.qj[d] = qn * b.scale[CH_JX + d];
+    for (int ch = 0; ch < 4; ++ch) {
+        k.mq[ch] = -b.m_cr * b.scale[ch];
+        k.vlim[ch] = (uint64_t)__double_as_longlong(b.qmax[ch] * b.scale[ch]);
+    }
+}
+
+// |q| > limit for the bits of a limit >= 0 (false for NaN)
+__device__ __forceinline__ bool beyond(double q, uint64_t limit)
+{
+    const uint64_t a = (uint64_t)__double_as_longlong(q) & 0x7fffffffffffffffull;
+    return a > limit && a <= 0x7ff0000000000000ull;
+}
+
 template <int D>
-__device__ __forceinline__ void gather_f64(const Ctx &c, const BoxDev &b, bool in_tile, const int rel[3],
-                                           const int ci[3], const double wx[3], const double wy[3],
-                                           const double wz[3], const double2 *__restrict__ sF,
+__device__ __forceinline__ void gather_f64(const Ctx &c, const BoxDev &b, bool in_tile, int base,
+                                           const int ci[3], const double w[3][3], const double2 *__restrict__ sF,
                                            double E[3], double Bf[3])
 {
     E[0] = E[1] = E[2] = Bf[0] = Bf[1] = Bf[2] = 0.0;
     const double2 *__restrict__ gF = reinterpret_cast<const double2 *>(c.f64);
+    const int SY = c.ts[1], SZ = c.ts[2];
     int gx[3], gy[3], gz[3];
-    stencil_coords<D>(b, ci, gx, gy, gz);
-    int base = (rel[0] - 1) + c.ts[1] * (rel[1] - 1) + c.ts[2] * (D == 3 ? rel[2] - 1 : 0);
+    if (!in_tile)
+        stencil_coords<D>(b, ci, gx, gy, gz);
+#pragma unroll 1
     for (int cz = 0; cz < (D == 3 ? 3 : 1); ++cz)
-        for (int cy = 0; cy < 3; ++cy)
+#pragma unroll
+        for (int cy = 0; cy < 3; ++cy) {
+            const double wyz = D == 3 ? w[1][cy] * w[2][cz] : w[1][cy];
+#pragma unroll
             for (int cx = 0; cx < 3; ++cx) {
-                double w = wx[cx] * wy[cy] * (D == 3 ? wz[cz] : 1.0);
-                double2 a0, a1, a2;
-                if (in_tile) {
-                    int s = base + cx + c.ts[1] * cy + c.ts[2] * cz;
-                    a0 = sF[3 * s];
-                    a1 = sF[3 * s + 1];
-                    a2 = sF[3 * s + 2];
-                } else {
-                    int64_t g = b.cell0 + ((int64_t)gz[cz] * b.n[1] + gy[cy]) * b.n[0] + gx[cx];
-                    a0 = __ldg(gF + 3 * g);
-                    a1 = __ldg(gF + 3 * g + 1);
-                    a2 = __ldg(gF + 3 * g + 2);
-                }
-                E[0] += w * a0.x;
-                E[1] += w * a0.y;
-                E[2] += w * a1.x;
-                Bf[0] += w * a1.y;
-                Bf[1] += w * a2.x;
-                Bf[2] += w * a2.y;
+                const double ww = w[0][cx] * wyz;
+                const double2 *f = sF + 3 * (base + cx + SY * cy + SZ * cz);
+                if (!in_tile)
+                    f = gF + 3 * (b.cell0 + ((int64_t)gz[cz] * b.n[1] + gy[cy]) * b.n[0] + gx[cx]);
+                const double2 a0 = f[0], a1 = f[1], a2 = f[2];
+                E[0] += ww * a0.x;
+                E[1] += ww * a0.y;
+                E[2] += ww * a1.x;
+                Bf[0] += ww * a1.y;
+                Bf[1] += ww * a2.x;
+                Bf[2] += ww * a2.y;
             }
+        }
 }
 
-// Deposit 4 pre-scaled quantities (channels ch0..ch0+3) with TSC weights.
+// Cell and offset of a position, and the offset's TSC weights as integers.
 template <int D>
-__device__ __forceinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in_tile, const int rel[3],
-                                             const int ci[3], const double wx[3], const double wy[3],
-                                             const double wz[3], const double q[4], int ch0,
+__device__ __forceinline__ void cell_of_f64(const F64Const &k, const double x[3], int ci[3], double o[3])
+{
+    // s + 1.5 2^52 rounded down holds floor(s) in its low word
+    constexpr double FLOOR = 6755399441055744.0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const double s = (x[d] - k.lo[d]) * k.inv_dx[d];
+        const double t = __dadd_rd(s, FLOOR);
+        ci[d] = __double2loint(t);
+        o[d] = s - (t - FLOOR);
+    }
+}
+
+// Four channels (already at their scales) with the TSC weights of offsets o:
+// into the tile when the stencil lies in it, else into the global
+// accumulators; the same integers either way.
+template <int D>
+__device__ __forceinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in_tile, int base, const int ci[3],
+                                             const double o[3], const double q[4],
                                              unsigned long long *__restrict__ sD,
                                              unsigned long long *__restrict__ gdst)
 {
-    const int S = c.tile_slots;
+    const int S = c.tile_slots, SY = c.ts[1], SZ = c.ts[2];
     const int64_t nc = c.nc;
-    int gx[3], gy[3], gz[3];
-    stencil_coords<D>(b, ci, gx, gy, gz);
-    int base = (rel[0] - 1) + c.ts[1] * (rel[1] - 1) + c.ts[2] * (D == 3 ? rel[2] - 1 : 0);
-    for (int cz = 0; cz < (D == 3 ? 3 : 1); ++cz)
+    uint64_t wz[3] = {0ull, 1ull << 63, 0ull}, pair[9], mag[4], sign[4];
+    {
+        uint64_t wx[3], wy[3];
+        wide_tsc(o[0], wx);
+        wide_tsc(o[1], wy);
+        if (D == 3)
+            wide_tsc(o[2], wz);
+#pragma unroll
         for (int cy = 0; cy < 3; ++cy)
-            for (int cx = 0; cx < 3; ++cx) {
-                double w = wx[cx] * wy[cy] * (D == 3 ? wz[cz] : 1.0);
-                if (in_tile) {
-                    int s = base + cx + c.ts[1] * cy + c.ts[2] * cz;
-                    for (int k = 0; k < 4; ++k)
-                        red_add(sD + (ch0 + k) * S + s, to_fixed(q[k] * w));
-                } else {
-                    int64_t g = b.cell0 + ((int64_t)gz[cz] * b.n[1] + gy[cy]) * b.n[0] + gx[cx];
-                    for (int k = 0; k < 4; ++k)
-                        red_add(gdst + k * nc + g, to_fixed(q[k] * w));
-                }
+#pragma unroll
+            for (int cx = 0; cx < 3; ++cx)
+                pair[3 * cy + cx] = wide_pair<WIDE>(wx[cx], wy[cy]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        wide_q<WIDE>(q[k], mag[k], sign[k]);
+    int gx[3], gy[3], gz[3];
+    if (!in_tile)
+        stencil_coords<D>(b, ci, gx, gy, gz);
+#pragma unroll 1
+    for (int cz = 0; cz < (D == 3 ? 3 : 1); ++cz) {
+        const uint64_t w = D == 3 ? (cz == 0 ? wz[0] : (cz == 1 ? wz[1] : wz[2])) : wz[1];
+        uint64_t qz[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            qz[k] = mul_hi_round(mag[k], w);
+        if (in_tile) {
+#pragma unroll
+            for (int n = 0; n < 9; ++n) {
+                unsigned long long *t = sD + base + n % 3 + SY * (n / 3) + SZ * cz;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    atomicAdd(t + k * S, wide_value(qz[k], pair[n], sign[k]));
             }
+        } else {
+#pragma unroll 1
+            for (int n = 0; n < 9; ++n) {
+                const int64_t g = b.cell0 + ((int64_t)gz[D == 3 ? cz : 1] * b.n[1] + gy[n / 3]) * b.n[0] + gx[n % 3];
+                uint64_t p = pair[0];
+#pragma unroll
+                for (int i = 1; i < 9; ++i)
+                    p = n == i ? pair[i] : p;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    atomicAdd(gdst + k * nc + g, wide_value(qz[k], p, sign[k]));
+            }
+        }
+    }
 }
 
-template <int D>
-__device__ __forceinline__ void cell_of_f64(const BoxDev &b, const double x[3], int ci[3], double w[3][3])
+// The particle boundary along d (boundary_f64): a particle inside a periodic
+// box, told by integer comparisons, only takes the rounding of x - lo + lo.
+__device__ __forceinline__ bool bounded(const BoxDev &b, const F64Const &k, int d, double &x, double &vd)
 {
-    for (int d = 0; d < D; ++d) {
-        double s = (x[d] - b.x0[d]) * b.inv_dx[d];
-        double f = floor(s);
-        ci[d] = (int)f;
-        tsc_from_offset<double>(s - f, w[d]);
+    if (b.bc[d] == MHDPIC_BC_PERIODIC) {
+        const double r = x - k.lo[d];
+        if ((uint64_t)__double_as_longlong(r) < (uint64_t)__double_as_longlong(k.L[d])) {
+            x = k.lo[d] + r;
+            return false;
+        }
     }
+    return boundary_f64(b, d, x, vd);
 }
 
 template <int D, bool FULL>
@@ -102,11 +199,12 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
                                               unsigned long long *sD, unsigned long long *mout)
 {
     const int64_t np = c.np;
-    const double C = k.C;
     const int64_t src = c.perm_src ? (int64_t)c.perm_src[j] : j;
     double x[3] = {0.0, 0.0, 0.0}, v[3];
+#pragma unroll
     for (int d = 0; d < D; ++d)
         x[d] = c.src_x[d * np + src];
+#pragma unroll
     for (int d = 0; d < 3; ++d)
         v[d] = c.src_p64[d * np + src];
     if (isnan(x[0])) {   // left the box earlier (kept until the next sort)
@@ -117,74 +215,95 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
         return 0.f;
     }
 
-    // a particle at an open face is held just inside it, deposits its
+    // gamma = sqrt(C^2 + v^2)/C and its inverse from one reciprocal square
+    // root; a particle at an open face is held just inside it, deposits its
     // corrector and then leaves
-    double g0 = sqrt(C * C + (v[0] * v[0] + v[1] * v[1] + v[2] * v[2])) / C;
+    const double s0 = k.C2 + (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+    const double y0 = reciprocal_sqrt(s0);
+    const double g0 = s0 * y0 * k.invC;
     bool leaving = false;
-    for (int d = 0; d < D; ++d) {
-        x[d] = x[d] + 0.5 * k.dt * (v[d] / g0);
-        leaving |= boundary_f64(b, d, x[d], v[d]);
+    {
+        const double hu = 0.5 * k.dt * (k.C * y0);
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            x[d] = x[d] + hu * v[d];
+            leaving |= bounded(b, k, d, x[d], v[d]);
+        }
     }
 
     int ci[3] = {0, 0, 0}, rel[3] = {0, 0, 0};
-    double w[3][3] = {{0, 1, 0}, {0, 1, 0}, {0, 1, 0}};
-    cell_of_f64<D>(b, x, ci, w);
+    double o[3];
+    cell_of_f64<D>(k, x, ci, o);
     bool in_tile = true;
+#pragma unroll
     for (int d = 0; d < D; ++d)
         in_tile &= tile_rel(c, b, gm, d, ci[d], rel[d]);
+    const int base = (rel[0] - 1) + c.ts[1] * (rel[1] - 1) + (D == 3 ? c.ts[2] * (rel[2] - 1) : 0);
 
     double E[3], Bf[3];
-    gather_f64<D>(c, b, in_tile, rel, ci, w[0], w[1], w[2], sF, E, Bf);
-    double B2 = Bf[0] * Bf[0] + Bf[1] * Bf[1] + Bf[2] * Bf[2];
+    {
+        double w[3][3];
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+            tsc_from_offset<double>(o[d], w[d]);
+        gather_f64<D>(c, b, in_tile, base, ci, w, sF, E, Bf);
+    }
+    const double B2 = Bf[0] * Bf[0] + Bf[1] * Bf[1] + Bf[2] * Bf[2];
     if (B2 > 0.0) {
-        double eb = (E[0] * Bf[0] + E[1] * Bf[1] + E[2] * Bf[2]) / B2;
+        const double eb = (E[0] * Bf[0] + E[1] * Bf[1] + E[2] * Bf[2]) * reciprocal(B2);
+#pragma unroll
         for (int d = 0; d < 3; ++d)
             E[d] -= eb * Bf[d];
     }
 
-    const double h = k.h;
-    double v0[3], v1[3], vn[3], bb[3], t[3], txb[3];
+    const double hh = 0.5 * k.h;
+    double e[3], v0[3], v1[3], vn[3], bb[3], t[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        e[d] = hh * E[d];
+        v0[d] = v[d] + e[d];
+    }
+    const double sm = k.C2 + (v0[0] * v0[0] + v0[1] * v0[1] + v0[2] * v0[2]);
+    const double ym = reciprocal_sqrt(sm);
+    const double gam = sm * ym * k.invC;
+    const double hb = hh * (k.C * ym);
+#pragma unroll
     for (int d = 0; d < 3; ++d)
-        v0[d] = v[d] + 0.5 * h * E[d];
-    double gam = sqrt(C * C + (v0[0] * v0[0] + v0[1] * v0[1] + v0[2] * v0[2])) / C;
+        bb[d] = hb * Bf[d];
+    t[0] = v0[0] + (v0[1] * bb[2] - v0[2] * bb[1]);
+    t[1] = v0[1] + (v0[2] * bb[0] - v0[0] * bb[2]);
+    t[2] = v0[2] + (v0[0] * bb[1] - v0[1] * bb[0]);
+    const double f = 2.0 * reciprocal(1.0 + (bb[0] * bb[0] + bb[1] * bb[1] + bb[2] * bb[2]));
+    v1[0] = v0[0] + f * (t[1] * bb[2] - t[2] * bb[1]);
+    v1[1] = v0[1] + f * (t[2] * bb[0] - t[0] * bb[2]);
+    v1[2] = v0[2] + f * (t[0] * bb[1] - t[1] * bb[0]);
+#pragma unroll
     for (int d = 0; d < 3; ++d)
-        bb[d] = 0.5 * h * Bf[d] / gam;
-    t[0] = v0[1] * bb[2] - v0[2] * bb[1];
-    t[1] = v0[2] * bb[0] - v0[0] * bb[2];
-    t[2] = v0[0] * bb[1] - v0[1] * bb[0];
-    for (int d = 0; d < 3; ++d)
-        t[d] += v0[d];
-    txb[0] = t[1] * bb[2] - t[2] * bb[1];
-    txb[1] = t[2] * bb[0] - t[0] * bb[2];
-    txb[2] = t[0] * bb[1] - t[1] * bb[0];
-    double b2 = bb[0] * bb[0] + bb[1] * bb[1] + bb[2] * bb[2];
-    for (int d = 0; d < 3; ++d)
-        v1[d] = v0[d] + 2.0 * txb[d] / (1.0 + b2);
-    for (int d = 0; d < 3; ++d)
-        vn[d] = v1[d] + 0.5 * h * E[d];
+        vn[d] = v1[d] + e[d];
 
     // dE_k: the rotation keeps |v|, so the energy change is that of the two
     // half kicks, E_k(a) - E_k(b) = (a-b).(a+b)/(gamma_a+gamma_b), a-b = (h/2)E
-    double g1 = sqrt(C * C + (vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2])) / C;
-    double dv[3], e[3], s1[3], s0[3];
-    for (int d = 0; d < 3; ++d) {
-        dv[d] = vn[d] - v[d];
-        e[d] = 0.5 * h * E[d];
-        s1[d] = vn[d] + v1[d];
-        s0[d] = v0[d] + v[d];
+    const double sn = k.C2 + (vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
+    const double yn = reciprocal_sqrt(sn);
+    const double g1 = sn * yn * k.invC, ig1 = k.C * yn;
+    const double dEk = (e[0] * (vn[0] + v1[0]) + e[1] * (vn[1] + v1[1]) + e[2] * (vn[2] + v1[2])) * reciprocal(g1 + gam) +
+                       (e[0] * (v0[0] + v[0]) + e[1] * (v0[1] + v[1]) + e[2] * (v0[2] + v[2])) * reciprocal(gam + g0);
+    {
+        const double qc[4] = {k.mq[0] * (vn[0] - v[0]), k.mq[1] * (vn[1] - v[1]), k.mq[2] * (vn[2] - v[2]),
+                              k.mq[3] * dEk};
+        if (beyond(qc[0], k.vlim[0]) || beyond(qc[1], k.vlim[1]) || beyond(qc[2], k.vlim[2]) ||
+            beyond(qc[3], k.vlim[3]))
+            set_status(c.status, MHDPIC_ST_OVERFLOW);
+        deposit4_f64<D>(c, b, in_tile, base, ci, o, qc, sD, c.corr);
     }
-    double dEk = (e[0] * s1[0] + e[1] * s1[1] + e[2] * s1[2]) / (g1 + gam) +
-                 (e[0] * s0[0] + e[1] * s0[1] + e[2] * s0[2]) / (gam + g0);
-    double qc[4] = {-k.m * dv[0] * k.scale[CH_MX], -k.m * dv[1] * k.scale[CH_MY],
-                    -k.m * dv[2] * k.scale[CH_MZ], -k.m * dEk * k.scale[CH_E]};
-    if (fabs(qc[0]) > k.vlim[CH_MX] || fabs(qc[1]) > k.vlim[CH_MY] || fabs(qc[2]) > k.vlim[CH_MZ] ||
-        fabs(qc[3]) > k.vlim[CH_E])
-        set_status(c.status, MHDPIC_ST_OVERFLOW);
-    deposit4_f64<D>(c, b, in_tile, rel, ci, w[0], w[1], w[2], qc, CH_MX, sD, c.corr);
 
-    for (int d = 0; d < D; ++d) {
-        x[d] = x[d] + 0.5 * k.dt * (vn[d] / g1);
-        leaving |= boundary_f64(b, d, x[d], vn[d]);
+    {
+        const double hu = 0.5 * k.dt * ig1;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            x[d] = x[d] + hu * vn[d];
+            leaving |= bounded(b, k, d, x[d], vn[d]);
+        }
     }
     leaving |= removed_early(c, j);
     if (leaving) {   // removed: no moments deposit; the next sort drops it
@@ -196,29 +315,31 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
         return 0.f;
     }
     if (FULL) {
-        int ci2[3] = {0, 0, 0}, rel2[3] = {0, 0, 0};
-        double w2[3][3] = {{0, 1, 0}, {0, 1, 0}, {0, 1, 0}};
-        cell_of_f64<D>(b, x, ci2, w2);
+        int rel2[3] = {0, 0, 0};
+        cell_of_f64<D>(k, x, ci, o);
         bool in2 = true;
+#pragma unroll
         for (int d = 0; d < D; ++d)
-            in2 &= tile_rel(c, b, gm, d, ci2[d], rel2[d]);
-        double qm[4];
-        qm[0] = k.qn * k.scale[CH_N];
-        for (int d = 0; d < 3; ++d)
-            qm[1 + d] = k.qn * (vn[d] / g1) * k.scale[CH_JX + d];
-        deposit4_f64<D>(c, b, in2, rel2, ci2, w2[0], w2[1], w2[2], qm, CH_N, sD, mout);
+            in2 &= tile_rel(c, b, gm, d, ci[d], rel2[d]);
+        const int base2 = (rel2[0] - 1) + c.ts[1] * (rel2[1] - 1) + (D == 3 ? c.ts[2] * (rel2[2] - 1) : 0);
+        const double qm[4] = {k.qn, k.qj[0] * (vn[0] * ig1), k.qj[1] * (vn[1] * ig1), k.qj[2] * (vn[2] * ig1)};
+        deposit4_f64<D>(c, b, in2, base2, ci, o, qm, sD + CH_N * c.tile_slots, mout);
     }
     if (!isfinite(vn[0] + vn[1] + vn[2]))
         set_status(c.status, MHDPIC_ST_NONFINITE);
+#pragma unroll
     for (int d = 0; d < D; ++d)
         c.x[d * np + j] = x[d];
+#pragma unroll
     for (int d = 0; d < 3; ++d)
         c.p64[d * np + j] = vn[d];
-    return (float)(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
+    // |v|^2 for the per-box maximum
+    const float f0 = (float)vn[0], f1 = (float)vn[1], f2 = (float)vn[2];
+    return f0 * f0 + f1 * f1 + f2 * f2;
 }
 
 template <int D, bool FULL>
-__global__ void __launch_bounds__(PUSH_THREADS) k_push_f64(Ctx c, const WorkItem *__restrict__ items,
+__global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkItem *__restrict__ items,
                                                           const int32_t *__restrict__ nitems,
                                                           int32_t *__restrict__ work_ctr, int cur_out,
                                                           double dt)
@@ -228,6 +349,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_f64(Ctx c, const WorkItem
     unsigned long long *sD = reinterpret_cast<unsigned long long *>(smem);
     double2 *sF = reinterpret_cast<double2 *>(smem + sizeof(unsigned long long) * NCH * S);
     __shared__ int s_item;
+    __shared__ F64Const s_k;
     unsigned long long *mout = c.momdep[cur_out];
     const int nit = *nitems;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -256,18 +378,11 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_f64(Ctx c, const WorkItem
             sF[3 * s + 1] = __ldg(gF + 3 * g + 1);
             sF[3 * s + 2] = __ldg(gF + 3 * g + 2);
         }
+        if (threadIdx.x == 0)
+            f64_const(b, dt, s_k);
         __syncthreads();
+        const F64Const &k = s_k;
 
-        F64Const k;
-        k.dt = dt;
-        k.h = b.qm_cr * dt;
-        k.C = b.C;
-        k.m = b.m_cr;
-        k.qn = b.qm_cr * b.m_cr * b.inv_dV;
-        for (int ch = 0; ch < NCH; ++ch) {
-            k.scale[ch] = b.scale[ch];
-            k.vlim[ch] = b.qmax[ch] * b.scale[ch];
-        }
         const LaneRange lr = lane_range(it, wid, NW);
         float vm2 = 0.f;
         for (int64_t r = lr.first; r < lr.q; r += lr.stride) {

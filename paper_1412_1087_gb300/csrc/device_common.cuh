@@ -129,12 +129,25 @@ __device__ __forceinline__ uint32_t res_pack(const int r[3])
     return ((uint32_t)r[0] & 0x3ffu) | (((uint32_t)r[1] & 0x3ffu) << 10) | (((uint32_t)r[2] & 0x3ffu) << 20);
 }
 
-// Exact double value of component d of a record.
+// Exact double value of component d of a record.  v[d] = m 2^(e-23) with a
+// 24-bit m, so the value is the whole number 1024 |m| +- r times 2^(e-33): put
+// together with integer operations and one FP64 subtraction (FP64 conversions
+// are as slow as FP64 arithmetic on this GPU); leading words below 2^-90,
+// infinities and NaN take the conversions.
 __device__ __forceinline__ double vel_f64(const float4 &w, int d)
 {
     const float h = d == 0 ? w.x : (d == 1 ? w.y : w.z);
     const int r = res_field(__float_as_uint(w.w), d);
-    return (double)h + (double)r * (double)res_quantum(res_exp(h));
+    const uint32_t b = __float_as_uint(h);
+    const int e = (int)((b >> 23) & 0xffu);
+    if (e < RES_EMIN + 127 || e == 255)
+        return (double)h + (double)r * (double)res_quantum(res_exp(h));
+    const uint32_t m = (b & 0x7fffffu) | 0x800000u;
+    const int rs = (int)b < 0 ? -r : r;
+    const uint64_t n = ((uint64_t)m << 10) + (uint64_t)(int64_t)rs;   // > 0, below 2^35
+    const double x = __hiloint2double(0x43300000 | (int)(n >> 32), (int)(uint32_t)n) - 4503599627370496.0;
+    const uint32_t hi = (uint32_t)__double2hiint(x) + ((uint32_t)(e - 127 - RES_SHIFT) << 20);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), __double2loint(x));
 }
 
 __device__ __forceinline__ void set_status(uint32_t *status, uint32_t flag)

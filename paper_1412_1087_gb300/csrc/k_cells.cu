@@ -2,6 +2,8 @@
 // cell-centred fields; the standalone charge/current deposit; FP64 totals;
 // read-back conversions.
 #include "cells_common.cuh"
+#include "math64.cuh"
+#include "wide_fixed.cuh"
 
 namespace mhdpic {
 
@@ -20,64 +22,48 @@ __global__ void k_scales(Ctx c, double dt)
     if (bx < c.nbox)
         scales_box(c, bx, dt);
 }
-// Charge and current densities at the current positions (App. A.1, eq:nJCR):
-// n = qm m W / dV, J = qm m u W / dV, straight into the global accumulators.
-template <int PREC, int D>
-__global__ void k_moments(Ctx c, int cur)
+// FP64 precision: charge and current densities at the current positions (App.
+// A.1, eq:nJCR), n = qm m W / dV, J = qm m u W / dV, straight into the global
+// accumulators, a warp's particles together (group_deposit).  Bound by the
+// FP64 pipe and the L2's 64-bit atomics.
+constexpr int MOMENTS_SH = 8;   // |q| scale <= 2^62 / (9 * 64): q 2^8 fits int64
+
+template <int D>
+__global__ void __launch_bounds__(256) k_moments_f64(Ctx c, int cur)
 {
-    unsigned long long *__restrict__ md = c.momdep[cur];
-    const int64_t nc = c.nc;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c.np;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (particle_dead<PREC>(c, i))   // left the box
-            continue;
-        int bx = find_box(c.box_part_start, c.nbox, i);
-        const BoxDev &b = c.boxes[bx];
-        int ci[3] = {0, 0, 0};
-        double w[3][3] = {{0, 1, 0}, {0, 1, 0}, {0, 1, 0}};
-        double v[3];
-        if (PREC == MHDPIC_PREC_MIXED) {
-            const int4 ps = c.pos[i];
-            const float4 vs = c.vel[i];
-            const float o[3] = {__int_as_float(ps.y), __int_as_float(ps.z), __int_as_float(ps.w)};
-            decode_cell(b, ps.x, ci);
+    __shared__ WideGroup<D> groups[256 / 32];
+    const int64_t np = c.np;
+    for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~31ll; i0 < np;
+         i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + (threadIdx.x & 31);
+        const bool live = i < np && !particle_dead<MHDPIC_PREC_FP64>(c, i);   // dead: left the box
+        double q[4], o[3];
+        int gx[3], gy[3], gz[3];
+        const BoxDev &b = c.boxes[find_box(c.box_part_start, c.nbox, i < np ? i : np - 1)];
+        if (live) {
+            int ci[3] = {0, 0, 0};
+#pragma unroll
             for (int d = 0; d < D; ++d)
-                tsc_from_offset<double>((double)o[d], w[d]);
+                floor_split((c.x[d * np + i] - b.x0[d]) * b.inv_dx[d], ci[d], o[d]);
+            double v[3];
+#pragma unroll
             for (int d = 0; d < 3; ++d)
-                v[d] = vel_f64(vs, d);
-        } else {
-            for (int d = 0; d < D; ++d) {
-                double s = (c.x[(int64_t)d * c.np + i] - b.x0[d]) * b.inv_dx[d];
-                double f = floor(s);
-                ci[d] = (int)f;
-                tsc_from_offset<double>(s - f, w[d]);
+                v[d] = c.p64[d * np + i];
+            const double ig = b.C * reciprocal_sqrt(b.C * b.C + (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]));
+            const double qn = b.qm_cr * b.m_cr * b.inv_dV;
+            q[0] = qn * b.scale[CH_N];
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                q[1 + d] = qn * b.scale[CH_JX + d] * (v[d] * ig);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                gx[a] = map_coord(ci[0] + a - 1, b.n[0], b.bc[0]);
+                gy[a] = map_coord(ci[1] + a - 1, b.n[1], b.bc[1]);
+                gz[a] = D == 3 ? map_coord(ci[2] + a - 1, b.n[2], b.bc[2]) : 0;
             }
-            for (int d = 0; d < 3; ++d)
-                v[d] = c.p64[(int64_t)d * c.np + i];
         }
-        double C = b.C;
-        double gam = sqrt(C * C + v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) / C;
-        double q[4];
-        q[0] = b.qm_cr * b.m_cr * b.inv_dV;
-        for (int d = 0; d < 3; ++d)
-            q[1 + d] = q[0] * (v[d] / gam);
-        for (int k = 0; k < 4; ++k)
-            q[k] *= b.scale[CH_N + k];
-        int gx[3], gy[3], gz[3] = {0, 0, 0};
-        for (int a = 0; a < 3; ++a) {
-            gx[a] = map_coord(ci[0] + a - 1, b.n[0], b.bc[0]);
-            gy[a] = map_coord(ci[1] + a - 1, b.n[1], b.bc[1]);
-            if (D == 3)
-                gz[a] = map_coord(ci[2] + a - 1, b.n[2], b.bc[2]);
-        }
-        for (int cz = 0; cz < (D == 3 ? 3 : 1); ++cz)
-            for (int cy = 0; cy < 3; ++cy)
-                for (int cxx = 0; cxx < 3; ++cxx) {
-                    double ww = w[0][cxx] * w[1][cy] * (D == 3 ? w[2][cz] : 1.0);
-                    int64_t gc = b.cell0 + ((int64_t)gz[cz] * b.n[1] + gy[cy]) * b.n[0] + gx[cxx];
-                    for (int k = 0; k < 4; ++k)
-                        red_add(md + k * nc + gc, to_fixed(q[k] * ww));
-                }
+        group_deposit<D, MOMENTS_SH>(groups[threadIdx.x >> 5], live, q, o, gx, gy, gz, b.cell0, b.n[0],
+                                     b.n[0] * b.n[1], c.momdep[cur], 1, c.nc);
     }
 }
 
@@ -270,18 +256,11 @@ int launch_moments(const Ctx &c, int cur, cudaStream_t st)
     cudaMemsetAsync(c.momdep[cur], 0, sizeof(unsigned long long) * 4 * c.nc, st);
     if (c.np == 0)
         return 0;
-    int g = grid_for(c.np, 256);
-    if (c.prec == MHDPIC_PREC_MIXED) {
-        if (c.ndim == 3)
-            k_moments<MHDPIC_PREC_MIXED, 3><<<g, 256, 0, st>>>(c, cur);
-        else
-            k_moments<MHDPIC_PREC_MIXED, 2><<<g, 256, 0, st>>>(c, cur);
-    } else {
-        if (c.ndim == 3)
-            k_moments<MHDPIC_PREC_FP64, 3><<<g, 256, 0, st>>>(c, cur);
-        else
-            k_moments<MHDPIC_PREC_FP64, 2><<<g, 256, 0, st>>>(c, cur);
-    }
+    const int g = grid_for(c.np, 256);
+    if (c.ndim == 3)
+        k_moments_f64<3><<<g, 256, 0, st>>>(c, cur);
+    else
+        k_moments_f64<2><<<g, 256, 0, st>>>(c, cur);
     return 1;
 }
 

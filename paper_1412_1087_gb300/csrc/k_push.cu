@@ -103,19 +103,13 @@ __device__ __forceinline__ void gather_f64(const Ctx &c, const BoxDev &b, bool i
         }
 }
 
-// Cell and offset of a position, and the offset's TSC weights as integers.
+// Cell and offset of a position.
 template <int D>
 __device__ __forceinline__ void cell_of_f64(const F64Const &k, const double x[3], int ci[3], double o[3])
 {
-    // s + 1.5 2^52 rounded down holds floor(s) in its low word
-    constexpr double FLOOR = 6755399441055744.0;
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        const double s = (x[d] - k.lo[d]) * k.inv_dx[d];
-        const double t = __dadd_rd(s, FLOOR);
-        ci[d] = __double2loint(t);
-        o[d] = s - (t - FLOOR);
-    }
+    for (int d = 0; d < D; ++d)
+        floor_split((x[d] - k.lo[d]) * k.inv_dx[d], ci[d], o[d]);
 }
 
 // Four channels (already at their scales) with the TSC weights of offsets o:

@@ -52,4 +52,14 @@ __device__ __forceinline__ double reciprocal_sqrt(double s)
     return fma(y, fma(e, 0.375, 0.5) * e, y);
 }
 
+// Whole part and rest of s, |s| < 2^31: s + 1.5 2^52 rounded down holds
+// floor(s) in its low word.
+__device__ __forceinline__ void floor_split(double s, int &whole, double &rest)
+{
+    constexpr double MAGIC_FLOOR = 6755399441055744.0;
+    const double t = __dadd_rd(s, MAGIC_FLOOR);
+    whole = __double2loint(t);
+    rest = s - (t - MAGIC_FLOOR);
+}
+
 }  // namespace mhdpic

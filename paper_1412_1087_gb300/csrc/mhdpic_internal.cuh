@@ -219,6 +219,7 @@ int launch_mark_free(const Ctx &c, const SortScratch &s, cudaStream_t st);
 int launch_count_live(const Ctx &c, unsigned long long *out, cudaStream_t st);
 int launch_vmax(const Ctx &c, cudaStream_t st);
 int launch_prep(const Ctx &c, int cur, int apply, cudaStream_t st);
+// FP64 precision: charge and current at the current positions into momdep[cur]
 int launch_moments(const Ctx &c, int cur, cudaStream_t st);
 int launch_push_mixed(const Ctx &c, const SortScratch &s, int32_t *work_ctr, int cur_out, int full,
                       double dt, int grid_blocks, cudaStream_t st);

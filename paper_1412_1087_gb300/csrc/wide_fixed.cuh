@@ -93,4 +93,71 @@ __device__ __forceinline__ unsigned long long wide_value(uint64_t qz, uint64_t p
     return (mul_hi_round(qz, pair) ^ sign) - sign;
 }
 
+// ---------------------------------------------------------------------------
+// A warp deposits 32 particles straight into global accumulators.  Each lane
+// prepares one particle; then 12 lanes of each half warp take one particle
+// together, a lane per x node and channel, so that the 64-bit atomics of one
+// instruction fall into few 32-byte sectors (what the L2 counts: 210e9 lane
+// atomics/s with a sector each, 650e9 with 12 neighbours).
+// ---------------------------------------------------------------------------
+template <int D>
+struct WideGroup {
+    static constexpr int YZ = D == 3 ? 9 : 3;
+    static constexpr int STRIDE = 33;   // one word beyond the lanes: no two rows on the same banks
+    int64_t q[4][STRIDE];
+    uint64_t wx[3][STRIDE];
+    uint64_t yz[YZ][STRIDE];
+    int32_t gx[3][STRIDE];
+    int32_t row[YZ][STRIDE];
+};
+
+// live: this lane has a particle, with quantities q at their scales, offset o
+// and stencil cells gx, gy, gz of a box whose first cell is cell0 and whose x
+// and x y extents are n0 and n01.  Cell c, channel k is acc[c cell_stride + k
+// chan_stride].  All lanes of the warp call it.
+template <int D, int SH, typename R>
+__device__ __forceinline__ void group_deposit(WideGroup<D> &s, bool live, const double q[4], const R o[3],
+                                              const int gx[3], const int gy[3], const int gz[3], int64_t cell0, int n0,
+                                              int n01, unsigned long long *__restrict__ acc, int64_t cell_stride,
+                                              int64_t chan_stride)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned mask = __ballot_sync(0xffffffffu, live);
+    if (live) {
+        uint64_t wx[3], wy[3], wz[3] = {0ull, 1ull << 63, 0ull};
+        wide_tsc(o[0], wx);
+        wide_tsc(o[1], wy);
+        if (D == 3)
+            wide_tsc(o[2], wz);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            s.q[k][lane] = __double2ll_rn(q[k] * (double)(1 << SH));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            s.wx[a][lane] = wx[a];
+            s.gx[a][lane] = gx[a];
+        }
+#pragma unroll
+        for (int n = 0; n < WideGroup<D>::YZ; ++n) {
+            s.yz[n][lane] = wide_pair<SH>(wy[n % 3], D == 3 ? wz[n / 3] : wz[1]);
+            s.row[n][lane] = (int32_t)(cell0 + gy[n % 3] * n0 + (D == 3 ? gz[n / 3] * n01 : 0));
+        }
+    }
+    __syncwarp();
+    const int r = lane & 15, cx = r >> 2, ch = r & 3;
+    for (int it = 0; it < 16; ++it) {
+        const int p = 2 * it + (lane >> 4);
+        if (r < 12 && ((mask >> p) & 1u)) {
+            const int64_t i = s.q[ch][p];
+            const uint64_t sign = (uint64_t)(i >> 63);
+            const uint64_t qx = mul_hi_round(((uint64_t)i ^ sign) - sign, s.wx[cx][p]);
+            unsigned long long *__restrict__ a = acc + s.gx[cx][p] * cell_stride + ch * chan_stride;
+#pragma unroll
+            for (int n = 0; n < WideGroup<D>::YZ; ++n)
+                atomicAdd(a + s.row[n][p] * cell_stride, wide_value(qx, s.yz[n][p], sign));
+        }
+    }
+    __syncwarp();
+}
+
 }  // namespace mhdpic

@@ -35,6 +35,18 @@ __device__ __forceinline__ int box_chunks(const BoxDev &b, int64_t per_chunk, in
     return (int)(k < 1 ? 1 : (k > nchunks ? nchunks : k));
 }
 
+// Sum of the n slices p[0], p[stride], ... by a warp: each lane adds every
+// 32nd in order, then the lanes in a fixed tree (the result in lane 0).
+__device__ __forceinline__ double sum_slices(const double *__restrict__ p, int n, int stride)
+{
+    double s = 0.0;
+    for (int k = threadIdx.x & 31; k < n; k += 32)
+        s += p[(int64_t)k * stride];
+    for (int o = 16; o > 0; o >>= 1)
+        s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // Map an unwrapped cell coordinate g along dimension d onto the box: periodic
 // wrap, or mirror fold at a reflecting wall (cell -1-k mirrors cell k); beyond
 // an open face the cells take the last cell's values (and deposits).

@@ -69,7 +69,9 @@ __global__ void __launch_bounds__(256) k_moments_f64(Ctx c, int cur)
 
 // Deterministic FP64 totals per box: block (chunk, box) reduces a fixed slice
 // of the box's cells and particles in a fixed order; a second kernel adds the
-// chunks in order.  out per box: P_gas(3), E_gas, P_CR(3), E_CR.
+// chunks in a fixed order.  out per box: P_gas(3), E_gas, P_CR(3), E_CR.  The
+// FP64 pipe bounds it: E_k from refined reciprocals (math64.cuh) instead of a
+// square root and two divisions.
 template <int PREC>
 __global__ void __launch_bounds__(256) k_totals_partial(Ctx c, int nchunks, int64_t per_chunk, double *partials)
 {
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(256) k_totals_partial(Ctx c, int nchunks, int6
     int64_t npb = b.part1 - b.part0;
     int64_t ps = (npb + nbc - 1) / nbc;
     int64_t p0 = b.part0 + chunk * ps, p1 = min(b.part1, p0 + ps);
+    const double C2 = b.C * b.C, invC = 1.0 / b.C, m_cr = b.m_cr;
     for (int64_t i = p0 + threadIdx.x; i < p1; i += blockDim.x) {
         double v[3];
         if (PREC == MHDPIC_PREC_MIXED) {
@@ -105,11 +108,12 @@ __global__ void __launch_bounds__(256) k_totals_partial(Ctx c, int nchunks, int6
             for (int d = 0; d < 3; ++d)
                 v[d] = c.p64[(int64_t)d * c.np + i];
         }
-        double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-        double gam = sqrt(b.C * b.C + v2) / b.C;
+        const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        const double s = C2 + v2;
         for (int d = 0; d < 3; ++d)
-            acc[4 + d] += b.m_cr * v[d];
-        acc[7] += b.m_cr * (v2 / (gam + 1.0));
+            acc[4 + d] += m_cr * v[d];
+        // E_k = v^2 / (gamma + 1)
+        acc[7] += m_cr * (v2 * reciprocal(fma(s * reciprocal_sqrt(s), invC, 1.0)));
     }
     __shared__ double red[8][256];
     for (int q = 0; q < 8; ++q)
@@ -125,16 +129,15 @@ __global__ void __launch_bounds__(256) k_totals_partial(Ctx c, int nchunks, int6
         partials[((int64_t)bx * nchunks + chunk) * 8 + threadIdx.x] = red[threadIdx.x][0];
 }
 
+// A warp per box and quantity sums the slices (sum_slices).
 __global__ void k_totals_final(int nbox, int nchunks, const double *partials, double *out)
 {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= nbox * 8)
         return;
-    int bx = t / 8, q = t % 8;
-    double s = 0.0;
-    for (int k = 0; k < nchunks; ++k)
-        s += partials[((int64_t)bx * nchunks + k) * 8 + q];
-    out[t] = s;
+    const double s = sum_slices(partials + (int64_t)(t / 8) * nchunks * 8 + t % 8, nchunks, 8);
+    if ((threadIdx.x & 31) == 0)
+        out[t] = s;
 }
 
 __global__ void k_fixed_to_double(Ctx c, const unsigned long long *__restrict__ src, int ch0,
@@ -271,7 +274,7 @@ int launch_totals(const Ctx &c, double *partials, int nchunks, int64_t per_chunk
         k_totals_partial<MHDPIC_PREC_MIXED><<<grid, 256, 0, st>>>(c, nchunks, per_chunk, partials);
     else
         k_totals_partial<MHDPIC_PREC_FP64><<<grid, 256, 0, st>>>(c, nchunks, per_chunk, partials);
-    k_totals_final<<<(c.nbox * 8 + 255) / 256, 256, 0, st>>>(c.nbox, nchunks, partials, out);
+    k_totals_final<<<c.nbox, 256, 0, st>>>(c.nbox, nchunks, partials, out);
     return 2;
 }
 

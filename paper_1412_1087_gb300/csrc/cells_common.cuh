@@ -4,6 +4,7 @@
 #pragma once
 
 #include "device_common.cuh"
+#include "math64.cuh"
 
 namespace mhdpic {
 
@@ -49,11 +50,12 @@ __device__ __forceinline__ void prep_cells(const Ctx &c, int cur, int apply)
         }
         double Bc[3] = {c.B[g], c.B[nc + g], c.B[2 * nc + g]};
         // FP64 divisions are slow on this GPU: the mixed path, whose fields
-        // are staged in FP32, divides once by rho (and once by n_g) and
-        // multiplies; the FP64 path keeps the oracle's divisions
+        // are staged in FP32, takes one refined reciprocal of rho (and of
+        // n_g and n_g + n) and multiplies; the FP64 path keeps the oracle's
+        // divisions
         double v[3];
         if (PREC == MHDPIC_PREC_MIXED) {
-            const double ir = 1.0 / rho;
+            const double ir = reciprocal(rho);
             v[0] = m[0] * ir;
             v[1] = m[1] * ir;
             v[2] = m[2] * ir;
@@ -70,10 +72,10 @@ __device__ __forceinline__ void prep_cells(const Ctx &c, int cur, int apply)
             double n = from_fixed(md[g], b.inv_scale[CH_N]);
             double J[3] = {from_fixed(md[nc + g], b.inv_scale[CH_JX]), from_fixed(md[2 * nc + g], b.inv_scale[CH_JY]),
                            from_fixed(md[3 * nc + g], b.inv_scale[CH_JZ])};
-            double R = n / (ng + n);
+            double R = PREC == MHDPIC_PREC_MIXED ? n * reciprocal(ng + n) : n / (ng + n);
             double JxB[3] = {J[1] * Bc[2] - J[2] * Bc[1], J[2] * Bc[0] - J[0] * Bc[2],
                              J[0] * Bc[1] - J[1] * Bc[0]};
-            const double ing = PREC == MHDPIC_PREC_MIXED ? 1.0 / ng : 0.0;
+            const double ing = PREC == MHDPIC_PREC_MIXED ? reciprocal(ng) : 0.0;
             for (int d = 0; d < 3; ++d) {
                 double F = (1.0 - R) * (n * E0[d] + JxB[d]);
                 E[d] = PREC == MHDPIC_PREC_MIXED ? E0[d] - F * ing : E0[d] - F / ng;

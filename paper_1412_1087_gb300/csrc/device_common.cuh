@@ -233,8 +233,25 @@ __device__ __forceinline__ int ghost_candidate(int k, int x, int n)
     return k == 0 ? x : (k <= FGHOST ? -k : n + (k - 1 - FGHOST));
 }
 
-__device__ __forceinline__ void store_fields_mixed(float4 *fa, float2 *fb, const BoxDev &b, int x, int y, int z,
-                                                   float4 a, float2 bb)
+// One dimension's padded positions of cell x: x itself, then the ghost below
+// and the ghost above that copy it (periodic or mirror image), as the first
+// two bits of the result tell; with -1 the candidates have to be tested one by
+// one (an open face's last cell, which several ghosts copy, and boxes narrower
+// than their ghosts).
+__device__ __forceinline__ int ghost_images(int x, int n, int pn, int bc, int u[3])
+{
+    const int top = pn - FGHOST;   // padded positions run up to here
+    const bool periodic = bc == MHDPIC_BC_PERIODIC;
+    u[0] = x;
+    u[1] = periodic ? x - n : -1 - x;
+    u[2] = periodic ? x + n : 2 * n - 1 - x;
+    if (n < FGHOST || top > 2 * n || (bc == MHDPIC_BC_WALL_OPEN && x == n - 1))
+        return -1;
+    return (u[1] >= -FGHOST ? 1 : 0) | (bc != MHDPIC_BC_WALL_OPEN && u[2] < top ? 2 : 0);
+}
+
+static __device__ __noinline__ void store_fields_any(float4 *fa, float2 *fb, const BoxDev &b, int x, int y, int z,
+                                              float4 a, float2 bb)
 {
     const int kx = 1 + FGHOST + (b.pn[0] - FGHOST - b.n[0]);
     const int ky = 1 + FGHOST + (b.pn[1] - FGHOST - b.n[1]);
@@ -256,6 +273,37 @@ __device__ __forceinline__ void store_fields_mixed(float4 *fa, float2 *fb, const
                 fb[f] = bb;
             }
         }
+    }
+}
+
+// Testing every candidate of every cell against the cell mapping made the
+// staging of a 26 x 22 x 30 box 25 us; most cells have no ghost at all.
+__device__ __forceinline__ void store_fields_mixed(float4 *fa, float2 *fb, const BoxDev &b, int x, int y, int z,
+                                                   float4 a, float2 bb)
+{
+    int ux[3], uy[3], uz[3];
+    const int mx = ghost_images(x, b.n[0], b.pn[0], b.bc[0], ux);
+    const int my = ghost_images(y, b.n[1], b.pn[1], b.bc[1], uy);
+    const int mz = b.ndim == 3 ? ghost_images(z, b.n[2], b.pn[2], b.bc[2], uz) : 0;
+    if ((mx | my | mz) < 0) {
+        store_fields_any(fa, fb, b, x, y, z, a, bb);
+        return;
+    }
+    const int64_t f0 = fidx(b, x, y, z);
+    fa[f0] = a;
+    fb[f0] = bb;
+    if ((mx | my | mz) == 0)
+        return;
+#pragma unroll 1
+    for (int t = 1; t < (b.ndim == 3 ? 27 : 9); ++t) {
+        const int iz = t / 9, iy = t / 3 % 3, ix = t % 3;
+        if ((ix && !((mx >> (ix - 1)) & 1)) || (iy && !((my >> (iy - 1)) & 1)) || (iz && !((mz >> (iz - 1)) & 1)))
+            continue;
+        const int64_t f = f0 + (ix == 1 ? ux[1] - x : (ix == 2 ? ux[2] - x : 0)) +
+                          (int64_t)(iy == 1 ? uy[1] - y : (iy == 2 ? uy[2] - y : 0)) * b.pn[0] +
+                          (int64_t)(iz == 1 ? uz[1] - z : (iz == 2 ? uz[2] - z : 0)) * b.pn[0] * b.pn[1];
+        fa[f] = a;
+        fb[f] = bb;
     }
 }
 

@@ -26,12 +26,14 @@
 // The gas energy takes only the CR sources (the paper's linear test gas is
 // isothermal, App. B.2).  All gas arithmetic is FP64.
 #include "device_common.cuh"
+#include "math64.cuh"
 
 namespace mhdpic {
 
 namespace {
 
 constexpr double FIXED_LIMIT_G = 4611686018427387904.0;  // 2^62
+constexpr int GAS_THREADS = 256;
 
 __device__ __forceinline__ void cross(const double a[3], const double b[3], double o[3])
 {
@@ -61,95 +63,122 @@ __device__ __forceinline__ void moments_at(const Ctx &c, const BoxDev &b, const 
     J[2] = from_fixed(md[3 * nc + g], b.inv_scale[CH_JZ]);
 }
 
-// F_CR (eq:lorentz2) and (1-R) J.E0 (eq:engeq) of one cell.
+// The CR sources at a cell and what the gas model takes from it: F_CR
+// (eq:lorentz2), (1-R) J.E0 (eq:engeq), the gas velocity, R, and 1/rho and
+// 1/n_g from refined reciprocals (FP64 divisions are slow on this GPU).
+struct CellForce {
+    double F[3], P, vg[3], oneR, irho, ing;
+};
+
 __device__ __forceinline__ void cr_force(const BoxDev &b, double rho, const double m[3], const double B[3], double n,
-                                         const double J[3], double F[3], double &P)
+                                         const double J[3], CellForce &f)
 {
-    // FP64 divisions are slow on this GPU: one reciprocal per cell
-    const double ir = 1.0 / rho;
-    const double vg[3] = {m[0] * ir, m[1] * ir, m[2] * ir};
+    f.irho = reciprocal(rho);
+    f.ing = 0.0;
+    f.oneR = 1.0;
+    if (b.hall) {
+        const double ng = b.qm_gas * rho;
+        f.ing = reciprocal(ng);
+        f.oneR = 1.0 - n * reciprocal(ng + n);
+    }
+    for (int d = 0; d < 3; ++d)
+        f.vg[d] = m[d] * f.irho;
     double vxb[3], JxB[3];
-    cross(vg, B, vxb);
+    cross(f.vg, B, vxb);
     const double E0[3] = {-vxb[0], -vxb[1], -vxb[2]};
-    const double R = b.hall ? n / (b.qm_gas * rho + n) : 0.0;
     cross(J, B, JxB);
     for (int d = 0; d < 3; ++d)
-        F[d] = (1.0 - R) * (n * E0[d] + JxB[d]);
-    P = (1.0 - R) * (J[0] * E0[0] + J[1] * E0[1] + J[2] * E0[2]);
+        f.F[d] = f.oneR * (n * E0[d] + JxB[d]);
+    f.P = f.oneR * (J[0] * E0[0] + J[1] * E0[1] + J[2] * E0[2]);
 }
 
-// CR-Hall field F_CR / n_g at cell g of the state (rho, mom, B) with moments md.
-__device__ __forceinline__ void hall_field(const Ctx &c, const BoxDev &b, const unsigned long long *md,
-                                           const double *rho, const double *mom, const double *B, int64_t g,
-                                           double H[3])
+// What a cell's x neighbours need of it: the transverse gas velocity and the
+// CR-Hall field F_CR / n_g.
+struct Neighbour {
+    double v[2], H[2];
+};
+
+__device__ __forceinline__ Neighbour neighbour_of(const CellForce &f)
+{
+    return {{f.vg[1], f.vg[2]}, {f.F[1] * f.ing, f.F[2] * f.ing}};
+}
+
+// The same from the state in memory (cells that another block holds).
+__device__ __noinline__ Neighbour neighbour_at(const Ctx &c, const BoxDev &b, const unsigned long long *md, int64_t g)
 {
     const int64_t nc = c.nc;
-    double n, J[3], F[3], P;
+    double n, J[3];
     moments_at(c, b, md, g, n, J);
-    const double m[3] = {mom[g], mom[nc + g], mom[2 * nc + g]};
-    const double Bc[3] = {B[g], B[nc + g], B[2 * nc + g]};
-    cr_force(b, rho[g], m, Bc, n, J, F, P);
-    const double ng = b.qm_gas * rho[g];
-    for (int d = 0; d < 3; ++d)
-        H[d] = F[d] / ng;
-}
-
-// Gas-model part of G at cell g of the state (rho, mom, B): dmom and dB
-// (without the CR-Hall curl, which the callers add).
-__device__ __forceinline__ void linear_x(const Ctx &c, const BoxDev &b, const double *rho, const double *mom,
-                                         const double *B, int64_t g, int64_t l, int64_t r, double dmom[3],
-                                         double dB[3])
-{
-    const int64_t nc = c.nc;
-    const double h = 0.5 * b.inv_dx[0];
-    const double Bx = B[g];
-    const double irr = 1.0 / rho[r], irl = 1.0 / rho[l];
-    dmom[0] = dB[0] = 0.0;
-    for (int d = 1; d < 3; ++d) {
-        dmom[d] = Bx * (B[d * nc + r] - B[d * nc + l]) * h;
-        dB[d] = Bx * (mom[d * nc + r] * irr - mom[d * nc + l] * irl) * h;
-    }
+    const double m[3] = {c.mom[g], c.mom[nc + g], c.mom[2 * nc + g]};
+    const double Bc[3] = {c.B[g], c.B[nc + g], c.B[2 * nc + g]};
+    CellForce f;
+    cr_force(b, c.rho[g], m, Bc, n, J, f);
+    return neighbour_of(f);
 }
 
 // Predictor: half state into `half` (planes rho, mom x3, egas, B x3) and the
 // cell fields of the half state (as the stage kernel: E0 = -v x B, with the
 // CR-Hall term E = E0 - F/n_g from the moments at x^n) for the push; clears
 // the moments buffer the next push fills; records max |E|, |B|.
+//
+// Bound by the FP64 pipe.  Each cell's force is formed once and its x
+// neighbours read it from shared memory (forming it for both neighbours too,
+// with divisions, took 190 us at 700 x 500).
 template <int PREC>
-__global__ void k_gas_predict(Ctx c, int cur, double dt, int model, double *__restrict__ half)
+__global__ void __launch_bounds__(GAS_THREADS) k_gas_predict(Ctx c, int cur, double dt, int model,
+                                                            double *__restrict__ half)
 {
+    __shared__ Neighbour nb[GAS_THREADS];
     const unsigned long long *__restrict__ md = c.momdep[cur];
     unsigned long long *__restrict__ mnext = c.momdep[cur ^ 1];
     const int64_t nc = c.nc;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < nc;
-         g += (int64_t)gridDim.x * blockDim.x) {
-        const int bx = find_box(c.box_cell_start, c.nbox, g);
+    // the loop is uniform over the block
+    for (int64_t g0 = blockIdx.x * (int64_t)GAS_THREADS; g0 < nc; g0 += (int64_t)gridDim.x * GAS_THREADS) {
+        const int64_t g = g0 + threadIdx.x;
+        const bool in = g < nc;
+        const int bx = in ? find_box(c.box_cell_start, c.nbox, g) : 0;
         const BoxDev &b = c.boxes[bx];
-        const double rho = c.rho[g];
-        const double m[3] = {c.mom[g], c.mom[nc + g], c.mom[2 * nc + g]};
-        const double Bc[3] = {c.B[g], c.B[nc + g], c.B[2 * nc + g]};
-        double n, J[3], F[3], P;
-        moments_at(c, b, md, g, n, J);
-        cr_force(b, rho, m, Bc, n, J, F, P);
+        double rho = 0.0, m[3], Bc[3], n = 0.0, J[3];
+        CellForce f;
+        if (in) {
+            rho = c.rho[g];
+            for (int d = 0; d < 3; ++d) {
+                m[d] = c.mom[d * nc + g];
+                Bc[d] = c.B[d * nc + g];
+            }
+            moments_at(c, b, md, g, n, J);
+            cr_force(b, rho, m, Bc, n, J, f);
+        }
         double dmom[3] = {0.0, 0.0, 0.0}, dB[3] = {0.0, 0.0, 0.0};
         if (model == MHDPIC_GAS_LINEAR_X) {
-            const int64_t l = x_neighbour(b, g, -1), r = x_neighbour(b, g, 1);
-            linear_x(c, b, c.rho, c.mom, c.B, g, l, r, dmom, dB);
-            if (b.hall) {
-                double Hl[3], Hr[3];
-                hall_field(c, b, md, c.rho, c.mom, c.B, l, Hl);
-                hall_field(c, b, md, c.rho, c.mom, c.B, r, Hr);
-                const double h = 1.0 / (2.0 * b.dx[0]);
-                dB[1] -= (Hr[2] - Hl[2]) * h;
-                dB[2] += (Hr[1] - Hl[1]) * h;
+            __syncthreads();   // the previous cells have been read
+            if (in)
+                nb[threadIdx.x] = neighbour_of(f);
+            __syncthreads();
+            if (in) {
+                const int64_t l = x_neighbour(b, g, -1), r = x_neighbour(b, g, 1);
+                const bool lin = l >= g0 && l < g0 + GAS_THREADS, rin = r >= g0 && r < g0 + GAS_THREADS;
+                const Neighbour L = lin ? nb[l - g0] : neighbour_at(c, b, md, l);
+                const Neighbour R = rin ? nb[r - g0] : neighbour_at(c, b, md, r);
+                const double h = 0.5 * b.inv_dx[0];
+                for (int d = 1; d < 3; ++d) {
+                    dmom[d] = Bc[0] * (c.B[d * nc + r] - c.B[d * nc + l]) * h;
+                    dB[d] = Bc[0] * (R.v[d - 1] - L.v[d - 1]) * h;
+                }
+                if (b.hall) {
+                    dB[1] -= (R.H[1] - L.H[1]) * h;
+                    dB[2] += (R.H[0] - L.H[0]) * h;
+                }
             }
         }
+        if (!in)
+            continue;
         double mh[3], Bh[3];
         for (int d = 0; d < 3; ++d) {
-            mh[d] = m[d] + 0.5 * dt * (dmom[d] - F[d]);
+            mh[d] = m[d] + 0.5 * dt * (dmom[d] - f.F[d]);
             Bh[d] = Bc[d] + 0.5 * dt * dB[d];
         }
-        const double egh = c.egas[g] - 0.5 * dt * P;
+        const double egh = c.egas[g] - 0.5 * dt * f.P;
         half[g] = rho;
         half[nc + g] = mh[0];
         half[2 * nc + g] = mh[1];
@@ -160,37 +189,36 @@ __global__ void k_gas_predict(Ctx c, int cur, double dt, int model, double *__re
         half[7 * nc + g] = Bh[2];
 
         // cell fields of the half state
-        const double irho = 1.0 / rho;
-        const double v[3] = {mh[0] * irho, mh[1] * irho, mh[2] * irho};
+        const double v[3] = {mh[0] * f.irho, mh[1] * f.irho, mh[2] * f.irho};
         const double E0[3] = {-(v[1] * Bh[2] - v[2] * Bh[1]), -(v[2] * Bh[0] - v[0] * Bh[2]),
                               -(v[0] * Bh[1] - v[1] * Bh[0])};
         double E[3] = {E0[0], E0[1], E0[2]};
         if (b.hall) {
-            const double ng = b.qm_gas * rho;
-            const double R = n / (ng + n);
             double JxB[3];
             cross(J, Bh, JxB);
-            for (int d = 0; d < 3; ++d) {
-                const double Fh = (1.0 - R) * (n * E0[d] + JxB[d]);
-                E[d] = E0[d] - Fh / ng;
-            }
+            const double w = f.oneR * f.ing;
+            for (int d = 0; d < 3; ++d)
+                E[d] = E0[d] - w * (n * E0[d] + JxB[d]);
         }
+        float em, bm;   // |E| and |B| for the per-box maxima
         if (PREC == MHDPIC_PREC_MIXED) {
             int ci[3];
             decode_cell(b, (int32_t)(g - b.cell0), ci);
-            store_fields_mixed(c.fa, c.fb, b, ci[0], ci[1], ci[2],
-                               make_float4((float)E[0], (float)E[1], (float)E[2], (float)Bh[0]),
-                               make_float2((float)Bh[1], (float)Bh[2]));
+            const float4 fa = make_float4((float)E[0], (float)E[1], (float)E[2], (float)Bh[0]);
+            const float2 fb = make_float2((float)Bh[1], (float)Bh[2]);
+            store_fields_mixed(c.fa, c.fb, b, ci[0], ci[1], ci[2], fa, fb);
+            em = sqrtf(fa.x * fa.x + fa.y * fa.y + fa.z * fa.z);
+            bm = sqrtf(fa.w * fa.w + fb.x * fb.x + fb.y * fb.y);
         } else {
-            double2 *f = reinterpret_cast<double2 *>(c.f64) + 3 * g;
-            f[0] = make_double2(E[0], E[1]);
-            f[1] = make_double2(E[2], Bh[0]);
-            f[2] = make_double2(Bh[1], Bh[2]);
+            double2 *q = reinterpret_cast<double2 *>(c.f64) + 3 * g;
+            q[0] = make_double2(E[0], E[1]);
+            q[1] = make_double2(E[2], Bh[0]);
+            q[2] = make_double2(Bh[1], Bh[2]);
+            em = (float)sqrt(E[0] * E[0] + E[1] * E[1] + E[2] * E[2]);
+            bm = (float)sqrt(Bh[0] * Bh[0] + Bh[1] * Bh[1] + Bh[2] * Bh[2]);
         }
         for (int q = 0; q < 4; ++q)
             mnext[q * nc + g] = 0ull;
-        const float em = (float)sqrt(E[0] * E[0] + E[1] * E[1] + E[2] * E[2]);
-        const float bm = (float)sqrt(Bh[0] * Bh[0] + Bh[1] * Bh[1] + Bh[2] * Bh[2]);
         const unsigned peers = __match_any_sync(__activemask(), bx);
         const unsigned eb = __reduce_max_sync(peers, __float_as_uint(em));
         const unsigned bb = __reduce_max_sync(peers, __float_as_uint(bm));
@@ -226,19 +254,22 @@ __global__ void k_gas_correct(Ctx c, double dt, int model, const double *__restr
         if (model == MHDPIC_GAS_LINEAR_X) {
             const int64_t l = x_neighbour(b, g, -1), r = x_neighbour(b, g, 1);
             const double *rho_h = half, *mom_h = half + nc, *B_h = half + 5 * nc;
-            linear_x(c, b, rho_h, mom_h, B_h, g, l, r, dmom, dB);
+            const double h = 0.5 * b.inv_dx[0], Bx = B_h[g];
+            const double irl = reciprocal(rho_h[l]), irr = reciprocal(rho_h[r]);
+            for (int d = 1; d < 3; ++d) {
+                dmom[d] = Bx * (B_h[d * nc + r] - B_h[d * nc + l]) * h;
+                dB[d] = Bx * (mom_h[d * nc + r] * irr - mom_h[d * nc + l] * irl) * h;
+            }
             if (b.hall) {
-                // F_CR = -dM / (dV dt), H = F_CR / n_g of the half state
-                double Hl[3], Hr[3];
-                for (int d = 0; d < 3; ++d) {
-                    Hl[d] = (-from_fixed(c.corr[d * nc + l], b.inv_scale[CH_MX + d]) / (b.dV * dt)) /
-                            (b.qm_gas * rho_h[l]);
-                    Hr[d] = (-from_fixed(c.corr[d * nc + r], b.inv_scale[CH_MX + d]) / (b.dV * dt)) /
-                            (b.qm_gas * rho_h[r]);
-                }
-                const double h = 1.0 / (2.0 * b.dx[0]);
-                dB[1] -= (Hr[2] - Hl[2]) * h;
-                dB[2] += (Hr[1] - Hl[1]) * h;
+                // F_CR = -dM / (dV dt), H = F_CR / n_g of the half state:
+                // H = corr (-inv_scale / (dV dt qm_gas)) / rho
+                const double k = -h * b.inv_dV * reciprocal(dt * b.qm_gas);
+                double dH[3];
+                for (int d = 1; d < 3; ++d)
+                    dH[d] = (from_fixed(c.corr[d * nc + r], b.inv_scale[CH_MX + d]) * irr -
+                             from_fixed(c.corr[d * nc + l], b.inv_scale[CH_MX + d]) * irl) * k;
+                dB[1] -= dH[2];
+                dB[2] += dH[1];
             }
         }
         for (int d = 0; d < 3; ++d) {

@@ -512,8 +512,9 @@ int mhdpic_run(mhdpic_ctx *ctx, double dt, int32_t nsteps, int32_t sort_every);
  * staging (and the gas copies of MHDPIC_MEM_HOST_GAS) on a second stream
  * beside the sort that follows the push, the two joined before the next
  * step; with enable == 0 they run in turn on the context's stream.  The
- * one-launch step applies to mixed precision with device buffers and no open
- * face or injection times (mhdpic_step_fusion tells whether it does); the
+ * one-launch step applies to mixed precision with device buffers, no open
+ * face or injection times and at most 524,288 particles, beyond which the
+ * separate launches are faster (mhdpic_step_fusion tells whether it does); the
  * results are the same bit for bit as those of mhdpic_interp_push(dt, 1)
  * followed by mhdpic_apply_feedback(NULL).  Each barrier waits at most one
  * second by default; a wait that runs out raises MHDPIC_ST_BARRIER (the step's

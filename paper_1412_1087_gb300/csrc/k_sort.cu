@@ -5,18 +5,22 @@
 // earlier ones.  Steps:
 //   1. key of each particle, rank among equal keys by warp-aggregated atomics
 //      (this rank is not yet the stable one);
-//   2. exclusive scan of the per-key counts;
-//   3. scatter of the particle indices to their key segment;
+//   2. exclusive scan of the per-key counts (one kernel up to 8 tiles of 4096
+//      keys, two beyond);
+//   3. scatter of the particle indices to their key segment and, in the same
+//      launch, the push work list;
 //   4. sort of each key segment by particle index, which makes the result the
 //      stable order: the permutation equals a stable sort by key.
 // The particle arrays are permuted later: by the next push, which reads its
 // particles through the permutation, or by launch_gather.
-//   5. the push work list: every brick's particle range cut into items of at
-//      most ITEM_MAX_PARTICLES.
+// The work list cuts every brick's particle range into items of at most
+// item_cap particles.  At 64^2 x 16 particles a sort is launches and latency:
+// 12 kernels and 5 memsets took 60 us, 5 kernels and one memset take 25.
 #include <climits>
 
 #include "async_copy.cuh"
 #include "device_common.cuh"
+#include "math64.cuh"
 
 namespace mhdpic {
 
@@ -170,17 +174,27 @@ __device__ __forceinline__ int32_t key_f64(const Ctx &c, const BoxDev &b, int bx
 {
     int ci[3] = {0, 0, 0};
     const bool ahead = c.sort_ahead != 0.0;
-    if (isnan(c.x[i]))   // particles that left the box share one key after all the others
+    double x[3];
+    for (int d = 0; d < c.ndim; ++d)
+        x[d] = c.x[(int64_t)d * c.np + i];
+    if (isnan(x[0]))   // particles that left the box share one key after all the others
         return (int32_t)c.nkeys;
     float o[3] = {0.f, 0.f, 0.f};
     for (int d = 0; d < c.ndim; ++d) {
-        double s = (c.x[(int64_t)d * c.np + i] - b.x0[d]) / b.dx[d];
-        double f = floor(s);
-        int v = f < 0.0 ? 0 : (f >= (double)b.n[d] ? b.n[d] - 1 : (int)f);
-        if (!(f >= 0.0 && f < (double)b.n[d]))
+        // dividing by a power of two is multiplying by its inverse, exactly
+        // (the FP64 pipe bounds this pass: 210 us at 48^3 x 16 with divisions
+        // and conversions to and from integers)
+        const bool pow2 = (__double_as_longlong(b.dx[d]) & 0xfffffffffffffll) == 0;
+        const double s = pow2 ? (x[d] - b.x0[d]) * b.inv_dx[d] : (x[d] - b.x0[d]) / b.dx[d];
+        if (s >= 0.0 && s < (double)b.n[d]) {
+            double rest;
+            floor_split(s, ci[d], rest);
+            o[d] = (float)rest;
+        } else {
             set_status(c.status, MHDPIC_ST_CELL_RANGE);
-        ci[d] = v;
-        o[d] = (float)(s - (double)v);
+            ci[d] = s >= (double)b.n[d] ? b.n[d] - 1 : 0;
+            o[d] = (float)(s - (double)ci[d]);
+        }
     }
     if (ahead) {
         const float v[3] = {(float)c.p64[i], (float)c.p64[c.np + i], (float)c.p64[2 * c.np + i]};
@@ -403,49 +417,54 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int *
     return pre;
 }
 
+// The thread's SCAN_PER_THREAD counts of one tile (zeros past the end).
+__device__ __forceinline__ int4 scan_load(const int32_t *__restrict__ in, int64_t base, int64_t n)
+{
+    static_assert(SCAN_PER_THREAD == 4, "one 16-byte load per thread");
+    if (base + 3 < n)
+        return __ldg(reinterpret_cast<const int4 *>(in + base));
+    int4 v = make_int4(0, 0, 0, 0);
+    if (base < n)
+        v.x = in[base];
+    if (base + 1 < n)
+        v.y = in[base + 1];
+    if (base + 2 < n)
+        v.z = in[base + 2];
+    return v;
+}
+
 __global__ void k_scan_tiles(const int32_t *__restrict__ in, int64_t n, int32_t *__restrict__ sums)
 {
     __shared__ int ws[32];
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER_THREAD;
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < SCAN_PER_THREAD; ++k)
-        if (base + k < n)
-            s += in[base + k];
+    const int4 v = scan_load(in, blockIdx.x * (int64_t)SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER_THREAD, n);
     int tot;
-    block_exclusive_scan(s, ws, &tot);
+    block_exclusive_scan(v.x + v.y + v.z + v.w, ws, &tot);
     if (threadIdx.x == 0)
         sums[blockIdx.x] = tot;
 }
 
-__global__ void k_scan_sums(int32_t *sums, int nt)
-{
-    __shared__ int ws[32];
-    int carry = 0;
-    for (int start = 0; start < nt; start += blockDim.x) {
-        int i = start + threadIdx.x;
-        int v = i < nt ? sums[i] : 0;
-        int tot;
-        int pre = block_exclusive_scan(v, ws, &tot);
-        if (i < nt)
-            sums[i] = pre + carry;
-        carry += tot;
-    }
-}
-
+// Exclusive scan of tile blockIdx.x.  What lies before it is the sum of the
+// tiles before, from `sums` or, with sums null, added up from the counts.
 __global__ void k_scan_apply(const int32_t *__restrict__ in, int64_t n,
                              const int32_t *__restrict__ sums, int32_t *__restrict__ out)
 {
     __shared__ int ws[32];
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER_THREAD;
-    int vals[SCAN_PER_THREAD];
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-        vals[k] = base + k < n ? in[base + k] : 0;
-        s += vals[k];
+    int before = 0;
+    if (sums) {
+        for (int t = threadIdx.x; t < (int)blockIdx.x; t += SCAN_THREADS)
+            before += sums[t];
+    } else {
+        for (int t = 0; t < (int)blockIdx.x; ++t) {
+            const int4 v = scan_load(in, t * (int64_t)SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER_THREAD, n);
+            before += v.x + v.y + v.z + v.w;
+        }
     }
-    int pre = block_exclusive_scan(s, ws, nullptr) + sums[blockIdx.x];
+    int carry;
+    block_exclusive_scan(before, ws, &carry);
+    const int64_t base = blockIdx.x * (int64_t)SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER_THREAD;
+    const int4 v = scan_load(in, base, n);
+    int pre = block_exclusive_scan(v.x + v.y + v.z + v.w, ws, nullptr) + carry;
+    const int vals[SCAN_PER_THREAD] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int k = 0; k < SCAN_PER_THREAD; ++k) {
         if (base + k < n)
@@ -457,27 +476,116 @@ __global__ void k_scan_apply(const int32_t *__restrict__ in, int64_t n,
         out[n] = pre;
 }
 
-// out[0..n] = exclusive scan of in[0..n), out[n] = total.
+// out[0..n] = exclusive scan of in[0..n), out[n] = total (n >= 1).  Up to
+// SCAN_DIRECT tiles each block adds up the counts of the tiles before its own
+// (one launch instead of three); beyond, a first launch sums the tiles and
+// each block adds up the sums before it, at 2 million keys 512 of them (at
+// most one load per thread up to 4 million keys, a few dozen at 134 million:
+// too little for a launch of its own).
+constexpr int SCAN_DIRECT = 8;
+
 int scan(const int32_t *in, int64_t n, int32_t *out, int32_t *tmp, cudaStream_t st)
 {
-    if (n <= 0) {
-        cudaMemsetAsync(out, 0, sizeof(int32_t), st);
-        return 0;
+    const int nt = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
+    if (nt <= SCAN_DIRECT) {
+        k_scan_apply<<<nt, SCAN_THREADS, 0, st>>>(in, n, nullptr, out);
+        return 1;
     }
-    int nt = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
     k_scan_tiles<<<nt, SCAN_THREADS, 0, st>>>(in, n, tmp);
-    k_scan_sums<<<1, SCAN_THREADS, 0, st>>>(tmp, nt);
     k_scan_apply<<<nt, SCAN_THREADS, 0, st>>>(in, n, tmp, out);
-    return 3;
+    return 2;
 }
 
-// A key outside [0, nkeys] (only after a key pass that gave up part of its
-// work) is flagged and its particle skipped.
-__global__ void k_sort_scatter(int64_t np, int64_t nkeys, const int32_t *__restrict__ pkey,
-                               const int32_t *__restrict__ pslot, const int32_t *__restrict__ offset,
-                               int32_t *__restrict__ perm, uint32_t *status)
+// Items of a brick of cnt particles, na of them in its first half.
+__device__ __forceinline__ int brick_items(const Ctx &c, int cnt, int na)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    if (cnt <= c.item_cap)
+        return cnt > 0 ? 1 : 0;
+    if (!c.halves)
+        return (cnt + c.item_cap - 1) / c.item_cap;
+    return (na + c.item_cap - 1) / c.item_cap + (cnt - na + c.item_cap - 1) / c.item_cap;
+}
+
+// The push work list, SORT_THREADS consecutive bricks per block and pass:
+// their items go to a range of the list that the block reserves (the order of
+// the ranges does not matter: the deposits are integer sums).
+constexpr int SORT_THREADS = 256;
+
+__device__ __forceinline__ void write_items(const Ctx &c, const int64_t *__restrict__ brick_start,
+                                            const int32_t *__restrict__ offset, WorkItem *__restrict__ items,
+                                            int32_t *__restrict__ nitems, int block, int nblocks)
+{
+    __shared__ int ws[32];
+    __shared__ int s_first;
+    const int vol = c.brick[0] * c.brick[1] * c.brick[2];
+    for (int64_t g0 = (int64_t)block * SORT_THREADS; g0 < c.nbricks_total; g0 += (int64_t)nblocks * SORT_THREADS) {
+        const int64_t gb = g0 + threadIdx.x;
+        WorkItem w;
+        int64_t pm = 0;
+        int m = 0;
+        if (gb < c.nbricks_total) {
+            w.box = find_box(brick_start, c.nbox, gb);
+            const BoxDev &b = c.boxes[w.box];
+            w.brick = (int32_t)(gb - b.brick0);
+            const int64_t k0 = b.key0 + (int64_t)w.brick * vol;
+            w.p0 = offset[k0];
+            w.p1 = offset[k0 + vol];
+            pm = c.halves ? (int64_t)offset[k0 + vol / 2] : w.p1;
+            m = brick_items(c, (int)(w.p1 - w.p0), (int)(pm - w.p0));
+        }
+        int tot;
+        const int pre = block_exclusive_scan(m, ws, &tot);
+        if (threadIdx.x == 0)
+            s_first = tot > 0 ? atomicAdd(nitems, tot) : 0;
+        __syncthreads();
+        int o = s_first + pre;
+        if (m > 0 && w.p1 - w.p0 <= c.item_cap) {
+            // one item; a whole 64-cell brick splits at its 32nd cell (the
+            // start of the second half)
+            w.pm = c.halves ? pm : -1;
+            w.step = 1;
+            w.count = (int32_t)(w.p1 - w.p0);
+            items[o] = w;
+        } else if (m > 0) {
+            // crowded: each part (the two halves, or the whole brick) into
+            // m_p interleaved items, item t taking positions t, t + m_p, ...
+            const int64_t lo[2] = {w.p0, pm}, hi[2] = {pm, w.p1};
+            for (int part = 0; part < 2; ++part) {
+                const int64_t n = hi[part] - lo[part];
+                const int mp = (int)((n + c.item_cap - 1) / c.item_cap);
+                for (int t = 0; t < mp; ++t) {
+                    w.p0 = lo[part] + t;
+                    w.p1 = hi[part];
+                    w.pm = -1;
+                    w.step = mp;
+                    w.count = (int32_t)((n - t + mp - 1) / mp);
+                    items[o++] = w;
+                }
+            }
+        }
+        __syncthreads();   // s_first and ws are free again
+    }
+}
+
+// Scatter (blocks below scatter_blocks) and the push work list (the blocks
+// after them); both need only the offsets.  A key outside [0, nkeys] (only
+// after a key pass that gave up part of its work) is flagged and its particle
+// skipped.
+__global__ void __launch_bounds__(SORT_THREADS) k_sort_scatter(Ctx c, const int64_t *__restrict__ brick_start,
+                                                               const int32_t *__restrict__ pkey,
+                                                               const int32_t *__restrict__ pslot,
+                                                               const int32_t *__restrict__ offset,
+                                                               int32_t *__restrict__ perm,
+                                                               WorkItem *__restrict__ items,
+                                                               int32_t *__restrict__ nitems, int scatter_blocks)
+{
+    if ((int)blockIdx.x >= scatter_blocks) {
+        write_items(c, brick_start, offset, items, nitems, blockIdx.x - scatter_blocks, gridDim.x - scatter_blocks);
+        return;
+    }
+    const int64_t np = c.np, nkeys = c.nkeys;
+    uint32_t *status = c.status;
+    const int64_t stride = (int64_t)scatter_blocks * blockDim.x;
     for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < np; i0 += SORT_ILP * stride) {
         int32_t key[SORT_ILP], slot[SORT_ILP];
 #pragma unroll
@@ -673,125 +781,141 @@ __device__ __forceinline__ bool warp_merge_runs(const int32_t *a, int n, int32_t
     return true;
 }
 
-// Segments of up to 128 are sorted in registers, up to WARP_SORT_MAX in the
-// warp's shared memory (by their runs when they have at most MERGE_RUNS, else
-// by a bitonic network); longer ones are listed for k_sort_big.  This sorts
-// one key's segment [s, s + n), read from perm (the warp's buffer a is free).
-__device__ __forceinline__ void sort_one_segment(int64_t k, int s, int n, int32_t *__restrict__ perm, int32_t *a,
-                                                 int *hp, int32_t *__restrict__ big_list,
-                                                 int32_t *__restrict__ big_count, int lane)
+// One segment [s, s + n) of 128 < n <= WARP_SORT_MAX by a warp, through its
+// shared-memory buffer: by its runs when they are at most MERGE_RUNS, else by
+// a bitonic network.
+__device__ __forceinline__ void sort_mid_segment(int s, int n, int32_t *__restrict__ perm, int32_t *a, int *hp,
+                                                 int lane)
+{
+    int P = 64;
+    while (P < n)
+        P <<= 1;
+    for (int i = lane; i < P; i += 32)
+        a[i] = i < n ? perm[s + i] : INT_MAX;
+    __syncwarp();
+    if (warp_merge_runs(a, n, perm, s, lane, hp))
+        return;
+    for (int kk = 2; kk <= P; kk <<= 1) {
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            for (int i = lane; i < P; i += 32) {
+                int ixj = i ^ j;
+                if (ixj > i) {
+                    int x = a[i], y = a[ixj];
+                    bool asc = (i & kk) == 0;
+                    if ((x > y) == asc) {
+                        a[i] = y;
+                        a[ixj] = x;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    for (int i = lane; i < n; i += 32)
+        perm[s + i] = a[i];
+    __syncwarp();
+}
+
+// A warp takes `group` consecutive keys (at most SEG_GROUP) at a time: their
+// offsets in one load (one per lane), and, when the group's particles fit the
+// warp's buffer, all of them in one coalesced pass, so that the loads of a
+// whole group are in flight together; each segment of up to 128 is then sorted
+// in registers.  Longer segments are listed for k_sort_long (crowded cells lie
+// side by side: sorted here, one warp would take all of a group's in turn):
+// up to WARP_SORT_MAX from the front of the list, the others from its end.
+constexpr int SEG_GROUP = 31;
+// Particles of a warp's buffer.  Its size lets 5 blocks of 8 warps share an SM,
+// not 6: 6 make the SM keep 228 KB as shared memory instead of 196, it stays so
+// when a push of another context starts on it (which needs less), and that
+// push has half the L1 for its particle records (3% of the 128^3 x 32 step
+// with three contexts at work; a stated split on every launch costs 1% where
+// one is).  k_sort_long likewise.
+constexpr int SEG_BUFFER = 1200;
+
+__device__ __forceinline__ void sort_short_segment(const int32_t *src, int32_t *__restrict__ perm, int s, int n,
+                                                   int lane)
 {
     if (n <= 1)
         return;
-    if (n <= 32) {
-        warp_sort_segment<1>(perm + s, perm, s, n, lane);
-    } else if (n <= 64) {
-        warp_sort_segment<2>(perm + s, perm, s, n, lane);
-    } else if (n <= 128) {
-        warp_sort_segment<4>(perm + s, perm, s, n, lane);
-    } else if (n <= WARP_SORT_MAX) {
-        int P = 64;
-        while (P < n)
-            P <<= 1;
-        for (int i = lane; i < P; i += 32)
-            a[i] = i < n ? perm[s + i] : INT_MAX;
-        __syncwarp();
-        if (warp_merge_runs(a, n, perm, s, lane, hp))
-            return;
-        for (int kk = 2; kk <= P; kk <<= 1) {
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                for (int i = lane; i < P; i += 32) {
-                    int ixj = i ^ j;
-                    if (ixj > i) {
-                        int x = a[i], y = a[ixj];
-                        bool asc = (i & kk) == 0;
-                        if ((x > y) == asc) {
-                            a[i] = y;
-                            a[ixj] = x;
-                        }
-                    }
-                }
-                __syncwarp();
-            }
-        }
-        for (int i = lane; i < n; i += 32)
-            perm[s + i] = a[i];
-        __syncwarp();
-    } else if (lane == 0) {
-        int slot = atomicAdd(big_count, 1);
-        big_list[slot] = (int32_t)k;
-    }
+    if (n <= 32)
+        warp_sort_segment<1>(src, perm, s, n, lane);
+    else if (n <= 64)
+        warp_sort_segment<2>(src, perm, s, n, lane);
+    else
+        warp_sort_segment<4>(src, perm, s, n, lane);
 }
 
-// A warp takes SEG_GROUP consecutive keys at a time: their offsets in one
-// load (one per lane), and, when the group's particles fit the warp's buffer,
-// all of them in one coalesced pass, so that the loads of a whole group are in
-// flight together; each segment of up to 128 is then sorted from the buffer.
-// Longer segments, and groups that do not fit, go through sort_one_segment.
-constexpr int SEG_GROUP = 31;
-
-__global__ void __launch_bounds__(256) k_sort_segments(int64_t nkeys, const int32_t *__restrict__ offset,
+__global__ void __launch_bounds__(256) k_sort_segments(int64_t nkeys, int group, const int32_t *__restrict__ offset,
                                                        int32_t *__restrict__ perm,
-                                                       int32_t *__restrict__ big_list,
-                                                       int32_t *__restrict__ big_count)
+                                                       int32_t *__restrict__ long_list,
+                                                       int32_t *__restrict__ long_count)
 {
-    __shared__ int32_t buf[8][WARP_SORT_MAX];
-    __shared__ int hp[8][MERGE_RUNS];
+    __shared__ int32_t buf[8][SEG_BUFFER];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t *a = buf[wid];
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t k0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * SEG_GROUP; k0 < nkeys;
-         k0 += nwarps * SEG_GROUP) {
-        const int nk = (int)(nkeys - k0 < SEG_GROUP ? nkeys - k0 : SEG_GROUP);
+    for (int64_t k0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + wid) * group; k0 < nkeys;
+         k0 += nwarps * group) {
+        const int nk = (int)(nkeys - k0 < group ? nkeys - k0 : group);
         const int o = lane <= nk ? offset[k0 + lane] : 0;   // offsets of keys k0 .. k0 + nk
         const int gs = __shfl_sync(0xffffffffu, o, 0), ge = __shfl_sync(0xffffffffu, o, nk);
-        if (ge - gs > WARP_SORT_MAX) {
-            for (int j = 0; j < nk; ++j) {
-                const int s = __shfl_sync(0xffffffffu, o, j), e = __shfl_sync(0xffffffffu, o, j + 1);
-                sort_one_segment(k0 + j, s, e - s, perm, a, hp[wid], big_list, big_count, lane);
-            }
-            continue;
+        const int len = __shfl_down_sync(0xffffffffu, o, 1) - o;
+        // the long segments of the group go to the list
+        const bool mid = lane < nk && len > 128 && len <= WARP_SORT_MAX, big = lane < nk && len > WARP_SORT_MAX;
+        const unsigned mids = __ballot_sync(0xffffffffu, mid), bigs = __ballot_sync(0xffffffffu, big);
+        if (mids | bigs) {
+            int at = 0;
+            if (lane == 0 && mids)
+                at = atomicAdd(long_count, __popc(mids));
+            if (lane == 1 && bigs)
+                at = atomicAdd(long_count + 1, __popc(bigs));
+            const int m0 = __shfl_sync(0xffffffffu, at, 0), b0 = __shfl_sync(0xffffffffu, at, 1);
+            const unsigned below = (1u << lane) - 1u;
+            if (mid)
+                long_list[m0 + __popc(mids & below)] = (int32_t)(k0 + lane);
+            if (big)
+                long_list[nkeys - (b0 + __popc(bigs & below))] = (int32_t)(k0 + lane);
         }
-        for (int i = lane; i < ge - gs; i += 32)
-            a[i] = perm[gs + i];
-        __syncwarp();
-        unsigned longer = 0u;   // keys of the group with segments over 128
-        for (int j = 0; j < nk; ++j) {
-            const int s = __shfl_sync(0xffffffffu, o, j), e = __shfl_sync(0xffffffffu, o, j + 1);
-            const int n = e - s;
-            if (n <= 1)
-                continue;
-            if (n <= 32)
-                warp_sort_segment<1>(a + (s - gs), perm, s, n, lane);
-            else if (n <= 64)
-                warp_sort_segment<2>(a + (s - gs), perm, s, n, lane);
-            else if (n <= 128)
-                warp_sort_segment<4>(a + (s - gs), perm, s, n, lane);
-            else
-                longer |= 1u << j;
+        unsigned todo = __ballot_sync(0xffffffffu, lane < nk && len > 1 && len <= 128);
+        const bool staged = ge - gs <= SEG_BUFFER;
+        if (staged && todo) {
+            for (int i = lane; i < ge - gs; i += 32)
+                a[i] = perm[gs + i];
+            __syncwarp();
+        }
+        for (; todo; todo &= todo - 1u) {
+            const int j = __ffs(todo) - 1;
+            const int s = __shfl_sync(0xffffffffu, o, j), n = __shfl_sync(0xffffffffu, len, j);
+            sort_short_segment(staged ? a + (s - gs) : perm + s, perm, s, n, lane);
         }
         __syncwarp();   // the buffer is free again
-        while (longer) {
-            const int j = __ffs(longer) - 1;
-            longer &= longer - 1u;
-            const int s = __shfl_sync(0xffffffffu, o, j), e = __shfl_sync(0xffffffffu, o, j + 1);
-            sort_one_segment(k0 + j, s, e - s, perm, a, hp[wid], big_list, big_count, lane);
-        }
     }
 }
 
-// Long segments: block bitonic sort in shared memory, or a quadratic ranking
-// (elements are distinct particle indices) through `scratch` beyond that.
-__global__ void __launch_bounds__(1024) k_sort_big(const int32_t *__restrict__ offset,
+// The listed segments: a warp each up to WARP_SORT_MAX (the buffers of the
+// block's 8 warps), then a block each: bitonic sort in shared memory up to
+// BLOCK_SORT_MAX, or a quadratic ranking (elements are distinct particle
+// indices) through `scratch` beyond that.
+__global__ void __launch_bounds__(256) k_sort_long(int64_t nkeys, const int32_t *__restrict__ offset,
                                                    int32_t *__restrict__ perm,
-                                                   const int32_t *__restrict__ big_list,
-                                                   const int32_t *__restrict__ big_count,
+                                                   const int32_t *__restrict__ long_list,
+                                                   const int32_t *__restrict__ long_count,
                                                    int32_t *__restrict__ scratch, uint32_t *status)
 {
-    __shared__ int32_t a[BLOCK_SORT_MAX];
-    const int nb = *big_count;
+    static_assert(BLOCK_SORT_MAX == 8 * WARP_SORT_MAX && SEG_BUFFER - WARP_SORT_MAX >= MERGE_RUNS,
+                  "one buffer, by warps or whole, and the warps' run lists after it");
+    __shared__ int32_t a[8 * SEG_BUFFER];
+    int *const hp = a + BLOCK_SORT_MAX + (threadIdx.x >> 5) * MERGE_RUNS;
+    const int nm = long_count[0], nb = long_count[1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int q = blockIdx.x * 8 + wid; q < nm; q += gridDim.x * 8) {
+        const int64_t k = long_list[q];
+        const int s = offset[k];
+        sort_mid_segment(s, offset[k + 1] - s, perm, a + wid * WARP_SORT_MAX, hp, lane);
+    }
+    __syncthreads();   // the warps' buffers are free
     for (int q = blockIdx.x; q < nb; q += gridDim.x) {
-        int64_t k = big_list[q];
+        const int64_t k = long_list[nkeys - q];
         int s = offset[k], e = offset[k + 1];
         int n = e - s;
         if (n <= BLOCK_SORT_MAX) {
@@ -875,82 +999,6 @@ __global__ void k_perm_out(int64_t np, const int32_t *__restrict__ perm, int64_t
         out[r] = perm[r];
 }
 
-// Items per brick: ceil(count / ITEM_MAX_PARTICLES) near-equal pieces.
-__global__ void k_brick_items(Ctx c, const int64_t *__restrict__ brick_start,
-                              const int32_t *__restrict__ offset, int32_t *__restrict__ nitems_of)
-{
-    int64_t nbt = c.nbricks_total;
-    int vol = c.brick[0] * c.brick[1] * c.brick[2];
-    for (int64_t gb = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gb < nbt;
-         gb += (int64_t)gridDim.x * blockDim.x) {
-        int bx = find_box(brick_start, c.nbox, gb);
-        const BoxDev &b = c.boxes[bx];
-        int64_t k0 = b.key0 + (gb - b.brick0) * vol;
-        const int cnt = offset[k0 + vol] - offset[k0];
-        if (cnt <= ITEM_MAX_PARTICLES) {
-            nitems_of[gb] = cnt > 0 ? 1 : 0;
-        } else if (c.halves) {
-            const int na = offset[k0 + vol / 2] - offset[k0];
-            nitems_of[gb] = (na + ITEM_MAX_PARTICLES - 1) / ITEM_MAX_PARTICLES +
-                            (cnt - na + ITEM_MAX_PARTICLES - 1) / ITEM_MAX_PARTICLES;
-        } else {
-            nitems_of[gb] = (cnt + ITEM_MAX_PARTICLES - 1) / ITEM_MAX_PARTICLES;
-        }
-    }
-}
-
-__global__ void k_write_items(Ctx c, const int64_t *__restrict__ brick_start,
-                              const int32_t *__restrict__ offset, const int32_t *__restrict__ nitems_of,
-                              const int32_t *__restrict__ item_off, WorkItem *__restrict__ items,
-                              int32_t *__restrict__ nitems)
-{
-    int64_t nbt = c.nbricks_total;
-    int vol = c.brick[0] * c.brick[1] * c.brick[2];
-    for (int64_t gb = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gb < nbt;
-         gb += (int64_t)gridDim.x * blockDim.x) {
-        int bx = find_box(brick_start, c.nbox, gb);
-        const BoxDev &b = c.boxes[bx];
-        int64_t k0 = b.key0 + (gb - b.brick0) * vol;
-        const int64_t p0 = offset[k0], p1 = offset[k0 + vol];
-        const int m = nitems_of[gb];
-        if (m == 0)
-            continue;
-        int64_t o = item_off[gb];
-        WorkItem w;
-        w.box = bx;
-        w.brick = (int32_t)(gb - b.brick0);
-        if (p1 - p0 <= ITEM_MAX_PARTICLES) {
-            // one item; a whole 64-cell brick splits at its 32nd cell (the
-            // start of the second half)
-            w.p0 = p0;
-            w.p1 = p1;
-            w.pm = c.halves ? (int64_t)offset[k0 + vol / 2] : -1;
-            w.step = 1;
-            w.count = (int32_t)(p1 - p0);
-            items[o] = w;
-        } else {
-            // crowded: each part (the two halves, or the whole brick) into
-            // m_p interleaved items, item t taking positions t, t + m_p, ...
-            const int64_t pm = c.halves ? (int64_t)offset[k0 + vol / 2] : p1;
-            const int64_t lo[2] = {p0, pm}, hi[2] = {pm, p1};
-            for (int part = 0; part < 2; ++part) {
-                const int64_t n = hi[part] - lo[part];
-                const int mp = (int)((n + ITEM_MAX_PARTICLES - 1) / ITEM_MAX_PARTICLES);
-                for (int t = 0; t < mp; ++t) {
-                    w.p0 = lo[part] + t;
-                    w.p1 = hi[part];
-                    w.pm = -1;
-                    w.step = mp;
-                    w.count = (int32_t)((n - t + mp - 1) / mp);
-                    items[o++] = w;
-                }
-            }
-        }
-        if (gb == nbt - 1)
-            *nitems = item_off[nbt];
-    }
-}
-
 __global__ void k_max_count(int64_t n, const int32_t *__restrict__ count, int32_t *out)
 {
     int m = 0;
@@ -1003,7 +1051,8 @@ int launch_sort(const Ctx &c, const SortScratch &s, int64_t *perm_out, int32_t *
                 cudaStream_t st)
 {
     int launches = 0;
-    cudaMemsetAsync(s.count, 0, sizeof(int32_t) * (c.nkeys + 2), st);
+    // the counts and, after them, the counters of this sort
+    cudaMemsetAsync(s.count, 0, sizeof(int32_t) * (c.nkeys + 2 + SORT_COUNTERS), st);
     if (c.np > 0) {
         if (c.prec == MHDPIC_PREC_MIXED) {
             const bool ahead = c.sort_ahead != 0.0;
@@ -1022,16 +1071,24 @@ int launch_sort(const Ctx &c, const SortScratch &s, int64_t *perm_out, int32_t *
     // key nkeys holds the particles that left the box: offset[nkeys] is the
     // number of live particles
     launches += scan(s.count, c.nkeys + 1, s.offset, s.scan_tmp, st);
+    const int sb = c.np > 0 ? grid_for(c.np, SORT_THREADS) : 0;
+    k_sort_scatter<<<sb + grid_for(c.nbricks_total, SORT_THREADS), SORT_THREADS, 0, st>>>(
+        c, s.brick_start, s.pkey, s.pslot, s.offset, s.perm, s.items, s.nitems, sb);
+    ++launches;
     if (c.np > 0) {
-        cudaMemsetAsync(s.perm, 0, sizeof(int32_t) * c.np, st);
-        k_sort_scatter<<<grid_for(c.np, 256), 256, 0, st>>>(c.np, c.nkeys, s.pkey, s.pslot, s.offset, s.perm,
-                                                           c.status);
-        cudaMemsetAsync(s.big_count, 0, sizeof(int32_t), st);
-        const int64_t nw = (c.nkeys + 8 * SEG_GROUP - 1) / (8 * SEG_GROUP);   // blocks of 8 warps
+        // as many keys per warp as keep every resident warp at work (5 blocks
+        // of 8 warps per SM), at most SEG_GROUP: at 4,096 keys one each, 4 us
+        // against 18 with 31
+        const int64_t fit = (c.nkeys + 152 * 40 - 1) / (152 * 40);
+        const int group = (int)(fit < SEG_GROUP ? (fit < 1 ? 1 : fit) : SEG_GROUP);
+        const int64_t nw = (c.nkeys + 8 * group - 1) / (8 * group);   // blocks of 8 warps
         int gb = (int)(nw < 152 * 16 ? (nw < 1 ? 1 : nw) : 152 * 16);
-        k_sort_segments<<<gb, 256, 0, st>>>(c.nkeys, s.offset, s.perm, s.big_list, s.big_count);
-        k_sort_big<<<152, 1024, 0, st>>>(s.offset, s.perm, s.big_list, s.big_count, s.pkey, c.status);
-        launches += 3;
+        k_sort_segments<<<gb, 256, 0, st>>>(c.nkeys, group, s.offset, s.perm, s.long_list, s.long_count);
+        // no more warps than segments of over 128 there can be
+        const int64_t lw = (c.np / 128 + 7) / 8;
+        k_sort_long<<<(int)(lw < 1 ? 1 : (lw < 152 * 5 ? lw : 152 * 5)), 256, 0, st>>>(
+            c.nkeys, s.offset, s.perm, s.long_list, s.long_count, s.pkey, c.status);
+        launches += 2;
         if (perm_out) {
             k_perm_out<<<grid_for(c.np, 256), 256, 0, st>>>(c.np, s.perm, perm_out);
             ++launches;
@@ -1039,16 +1096,6 @@ int launch_sort(const Ctx &c, const SortScratch &s, int64_t *perm_out, int32_t *
     }
     if (counts_out)
         cudaMemcpyAsync(counts_out, s.count, sizeof(int32_t) * c.nkeys, cudaMemcpyDeviceToDevice, st);
-    // work list
-    const int64_t *brick_start = s.brick_start;
-    int32_t *nitems_of = s.brick_items;
-    int32_t *item_off = s.item_off;
-    int gb = grid_for(c.nbricks_total, 256);
-    k_brick_items<<<gb, 256, 0, st>>>(c, brick_start, s.offset, nitems_of);
-    launches += 1 + scan(nitems_of, c.nbricks_total, item_off, s.scan_tmp, st);
-    cudaMemsetAsync(s.nitems, 0, sizeof(int32_t), st);
-    k_write_items<<<gb, 256, 0, st>>>(c, brick_start, s.offset, nitems_of, item_off, s.items, s.nitems);
-    ++launches;
     return launches;
 }
 

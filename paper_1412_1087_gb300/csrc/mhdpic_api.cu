@@ -505,9 +505,6 @@ int do_sort(mhdpic_ctx *c, int64_t *perm_out, int32_t *counts_out)
     if ((rc = check_launch(c, launch_sort(c->k, c->s, perm_out, counts_out, c->stream))))
         return rc;
     c->pending = true;
-    // refresh the densest-cell count used by the corrector scales
-    if ((rc = check_launch(c, launch_max_count(c->k, c->s, c->stream))))
-        return rc;
     if (c->mem == MHDPIC_MEM_HOST && (rc = materialize(c)))
         return rc;
     return copy_particles(c, false);
@@ -529,8 +526,7 @@ int deposit_current(mhdpic_ctx *c, bool listed)
     Ctx kk = c->k;
     if (!listed) {
         if (!c->pending) {
-            if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))) ||
-                (rc = check_launch(c, launch_max_count(c->k, c->s, c->stream))))
+            if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))))
                 return rc;
             c->pending = true;
         }
@@ -739,8 +735,21 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
     if (k.nkeys >= 0x7fffffffLL)
         return bail(fail(MHDPIC_E_CAPACITY, "%lld sort keys exceed 2^31", (long long)k.nkeys));
 
-    // device allocations
     const int64_t np = k.np, nc = k.nc;
+    int bps = k.prec == MHDPIC_PREC_MIXED ? push_blocks_per_sm_mixed(k) : push_blocks_per_sm_f64(k);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    c->grid_blocks = bps * (nsm > 0 ? nsm : 1);
+    // work items: a brick's particles, but no more than there are for each
+    // resident block where that is less than a brick (small boxes leave SMs
+    // idle otherwise: 64 bricks of 1,024 particles at 64^2 x 16), in whole
+    // rounds of the block's threads
+    k.item_cap = (int32_t)std::min<int64_t>(
+        ITEM_MAX_PARTICLES,
+        std::max<int64_t>(1, (np / c->grid_blocks + PUSH_THREADS - 1) / PUSH_THREADS) * PUSH_THREADS);
+
+    // device allocations
     BoxDev *boxes_d;
     int64_t *ps_d, *cs_d;
     if ((rc = c->alloc(&boxes_d, nbox)) || (rc = c->alloc(&ps_d, nbox + 1)) || (rc = c->alloc(&cs_d, nbox + 1)) ||
@@ -770,20 +779,19 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
         if ((rc = setup_tensor_maps(c)))
             return bail(rc);
     }
-    int64_t scan_n = std::max<int64_t>(k.nkeys, k.nbricks_total) / 4096 + 2;
-    if ((rc = c->alloc(&c->s.count, k.nkeys + 2)) || (rc = c->alloc(&c->s.offset, k.nkeys + 2)) ||
+    const int64_t scan_n = k.nkeys / 4096 + 2;
+    if ((rc = c->alloc(&c->s.count, k.nkeys + 2 + SORT_COUNTERS)) || (rc = c->alloc(&c->s.offset, k.nkeys + 2)) ||
         (rc = c->alloc(&c->s.pkey, np)) || (rc = c->alloc(&c->s.pslot, np)) || (rc = c->alloc(&c->s.perm, np)) ||
-        (rc = c->alloc(&c->s.scan_tmp, scan_n)) || (rc = c->alloc(&c->s.big_list, k.nkeys + 1)) ||
-        (rc = c->alloc(&c->s.big_count, 1)) ||
+        (rc = c->alloc(&c->s.scan_tmp, scan_n)) || (rc = c->alloc(&c->s.long_list, k.nkeys + 1)) ||
         (rc = c->alloc((char **)&c->s.tmp, (size_t)np * c->particle_bytes())) ||
-        (rc = c->alloc(&c->s.brick_items, k.nbricks_total + 1)) ||
-        (rc = c->alloc(&c->s.item_off, k.nbricks_total + 1)) ||
         // at most one item per brick, or per half of a crowded brick
-        // ceil(n_half / ITEM_MAX_PARTICLES) <= n_half / ITEM_MAX_PARTICLES + 1
-        (rc = c->alloc(&c->s.items, 2 * k.nbricks_total + np / ITEM_MAX_PARTICLES + 2)) ||
-        (rc = c->alloc(&c->s.nitems, 1)) || (rc = c->alloc(&c->s.max_count, 1)) ||
+        // ceil(n_half / item_cap) <= n_half / item_cap + 1
+        (rc = c->alloc(&c->s.items, 2 * k.nbricks_total + np / k.item_cap + 2)) ||
+        (rc = c->alloc(&c->s.max_count, 1)) ||
         (rc = c->alloc(&c->work_ctr, 1)))
         return bail(rc);
+    c->s.long_count = c->s.count + k.nkeys + 2;
+    c->s.nitems = c->s.long_count + 2;
     k.key_off = c->s.offset;
     // chunked reductions (totals, spectrum): about 8 blocks per SM over all
     // boxes, each box sliced in proportion to its particles and cells
@@ -893,11 +901,6 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
         cudaStreamSynchronize(st))
         return bail(cuda_fail(cudaGetLastError(), "init stats"));
 
-    int bps = k.prec == MHDPIC_PREC_MIXED ? push_blocks_per_sm_mixed(k) : push_blocks_per_sm_f64(k);
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    c->grid_blocks = bps * (nsm > 0 ? nsm : 1);
     if (k.prec == MHDPIC_PREC_MIXED) {
         int coop = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -991,8 +994,7 @@ int mhdpic_interp_push(mhdpic_ctx *c, double dt, int32_t nsub)
         }
         // re-sort between sub-steps (the next sub-step applies it)
         if (!last && c->sub_sort_every > 0 && (s + 1) % c->sub_sort_every == 0) {
-            if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))) ||
-                (rc = check_launch(c, launch_max_count(c->k, c->s, c->stream))))
+            if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))))
                 return rc;
             c->pending = true;
         }
@@ -1075,8 +1077,7 @@ int mhdpic_inject(mhdpic_ctx *c, double dt, double eta, double energy_factor, do
     ++c->inj_calls;
     c->fields_stale = true;   // the compensation changed the gas
     // the new particles into their cells
-    if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))) ||
-        (rc = check_launch(c, launch_max_count(c->k, c->s, c->stream))))
+    if ((rc = check_launch(c, launch_sort(c->k, c->s, nullptr, nullptr, c->stream))))
         return rc;
     std::vector<unsigned char> img(inject_state_bytes());
     CK(cudaMemcpyAsync(img.data(), c->inj_state, img.size(), cudaMemcpyDeviceToHost, c->stream));
@@ -1363,11 +1364,18 @@ namespace {
 // The one-launch step applies where the step is exactly a push and a
 // feedback on device buffers: mixed precision, no open face (whose push is
 // followed by the marking of free slots), no injection times (their clock
-// and permutation are extra launches).
+// and permutation are extra launches).  And up to this many particles: the
+// cooperative launch needs the whole GPU to itself and its staging phase runs
+// at the push's occupancy, which outweighs the launches it saves (8 steps of
+// 1,048,576 particles 1003 us in one launch each and 985 apart, with two other
+// contexts at work 987 and 702; of 44.8 million 20.67 and 20.49 ms, 21.5 and
+// 19.97).
+constexpr int64_t FUSE_MAX_PARTICLES = 1 << 19;
+
 bool fused_ok(const mhdpic_ctx *c)
 {
     return c->fuse && c->step_grid > 0 && c->k.prec == MHDPIC_PREC_MIXED && c->mem == MHDPIC_MEM_DEVICE &&
-           !c->has_open && !c->track_tinj && c->k.np > 0;
+           !c->has_open && !c->track_tinj && c->k.np > 0 && c->k.np <= FUSE_MAX_PARTICLES;
 }
 
 // mhdpic_interp_push(dt, 1) + mhdpic_apply_feedback(NULL) as one cooperative

@@ -102,7 +102,7 @@ struct BoxStats {
 };
 
 // A work item: the sorted positions p0, p0 + step, ... below p1, all in one
-// brick.  A brick of at most ITEM_MAX_PARTICLES is one item of step 1; when
+// brick.  A brick of at most item_cap (<= ITEM_MAX_PARTICLES) is one item of step 1; when
 // it is a whole 64-cell brick, [p0, pm) and [pm, p1) are its two 32-cell
 // halves (one lane per cell), otherwise pm = -1.  A crowded brick becomes m
 // interleaved items per half (per brick without halves), item t taking the
@@ -113,7 +113,7 @@ struct WorkItem {
     int32_t brick;   // brick number inside the box
     int64_t p0, pm, p1;
     int32_t step;
-    int32_t count;   // positions in the item: ceil((p1 - p0) / step) <= ITEM_MAX_PARTICLES
+    int32_t count;   // positions in the item: ceil((p1 - p0) / step) <= item_cap
 };
 
 // Everything a kernel needs, passed by value.
@@ -128,6 +128,7 @@ struct Ctx {
     int32_t fts[3];        // field tile strides (x 1, y ts[1], z dense): the layout a tensor copy writes
     int32_t ftile_slots;   // slots of the field tile
     int32_t tma;           // 1: field tiles staged by tensor copies (tmaps), 0: by the threads
+    int32_t item_cap;      // particles of a work item, at most
     int32_t halves;        // 1: default 64-cell bricks split into 32-cell halves
     double sort_ahead;     // sort key: the cell after moving for this time at the current velocity
     const float4 *sort_k;  // per box {t/dx, t/dy, t/dz, 1/C^2} in FP32 for that key
@@ -176,18 +177,17 @@ struct Ctx {
 // launchers (each returns the number of kernel launches it made, or -1 on a
 // launch error; the caller checks cudaGetLastError)
 // ---------------------------------------------------------------------------
+constexpr int SORT_COUNTERS = 3;   // counters kept after the counts, cleared with them
 struct SortScratch {
-    int32_t *count;     // [nkeys + 1]
+    int32_t *count;     // [nkeys + 2], then long_count and nitems
     int32_t *offset;    // [nkeys + 1]
     int32_t *pkey;      // [np]
     int32_t *pslot;     // [np]
     int32_t *perm;      // [np]
     int32_t *scan_tmp;  // block sums
-    int32_t *big_list;  // segments longer than a warp can sort
-    int32_t *big_count; // [1]
+    int32_t *long_list;  // keys of segments longer than the segment pass sorts
+    int32_t *long_count; // [2] those a warp sorts, from the list's front, and those a block sorts, from its end
     void *tmp;          // particle staging, np * (largest particle record)
-    int32_t *brick_items;  // [nbricks + 1] items per brick
-    int32_t *item_off;     // [nbricks + 1] exclusive scan of brick_items
     int64_t *brick_start;  // device [nbox + 1] first global brick of each box
     WorkItem *items;
     int32_t *nitems;       // [1]

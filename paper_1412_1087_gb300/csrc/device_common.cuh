@@ -55,7 +55,10 @@ __device__ __forceinline__ int map_coord(int g, int n, int bc)
     if (bc == MHDPIC_BC_PERIODIC) {
         if (g >= 0 && g < n)
             return g;
-        int r = g % n;
+        int r = g < 0 ? g + n : g - n;   // one wrap, but for boxes narrower than their ghosts
+        if (r >= 0 && r < n)
+            return r;
+        r = g % n;
         return r < 0 ? r + n : r;
     }
     if (bc == MHDPIC_BC_WALL_OPEN) {
@@ -99,9 +102,8 @@ __device__ __forceinline__ int res_exp(float h)
     return e < RES_EMIN ? RES_EMIN : e;
 }
 
-// 2^(e - 33) and 2^(33 - e) for e in [RES_EMIN, 127]: both normal floats
+// 2^(e - 33) for e in [RES_EMIN, 127]: a normal float
 __device__ __forceinline__ float res_quantum(int e) { return __int_as_float((e - RES_SHIFT + 127) << 23); }
-__device__ __forceinline__ float res_inv_quantum(int e) { return __int_as_float((RES_SHIFT - e + 127) << 23); }
 
 __device__ __forceinline__ int res_field(uint32_t w, int d)
 {
@@ -120,20 +122,26 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &t)
 // (hi, r) += d: the exact sum hi + r q + d is rounded once, to the nearest
 // number the record can hold (34 significant bits).  TwoSum gives the
 // leading word and the exact remainder; the remainder is quantised to the
-// new word's residual grid.
+// new word's residual grid.  The exponents stay in place in the words (the
+// residual's unit and its inverse are integer sums of them), and r goes to
+// and from float through a magic sum: no conversions.
 __device__ __forceinline__ void two_word_add(float &hi, int &r, float d)
 {
-    const float rv = __fmul_rn((float)r, res_quantum(res_exp(hi)));   // exact
+    constexpr float MAGIC_R = 12582912.0f;   // 1.5 * 2^23
+    constexpr int MAGIC_R_BITS = 0x4B400000;
+    constexpr int E_MIN = (RES_EMIN + 127) << 23;
+    constexpr uint32_t E_SHIFT = (uint32_t)RES_SHIFT << 23;
+    const int e1 = max(__float_as_int(hi) & 0x7f800000, E_MIN);
+    const float rv = __fmul_rn(__fsub_rn(__int_as_float(MAGIC_R_BITS + r), MAGIC_R), __uint_as_float((uint32_t)e1 - E_SHIFT));
     float s, t;
     two_sum(hi, d, s, t);
     const float rem = __fadd_rn(t, rv);
     float h2, rem2;
     two_sum(s, rem, h2, rem2);
-    const int e2 = res_exp(h2);
-    const float q = rintf(__fmul_rn(rem2, res_inv_quantum(e2)));
-    const int qi = q > (float)RES_QMAX ? RES_QMAX : (q < -(float)RES_QMAX ? -RES_QMAX : (int)q);
+    const int e2 = max(__float_as_int(h2) & 0x7f800000, E_MIN);
+    const float q = __fadd_rn(__fmul_rn(rem2, __uint_as_float((254u << 23) + E_SHIFT - (uint32_t)e2)), MAGIC_R);
     hi = h2;
-    r = isfinite(h2) ? qi : 0;
+    r = max(-RES_QMAX, min(RES_QMAX, __float_as_int(q) - MAGIC_R_BITS));   // |q| is far below 2^22
 }
 
 __device__ __forceinline__ uint32_t res_pack(const int r[3])

@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
             sD[s] = 0ull;
         const double2 *gF = reinterpret_cast<const double2 *>(c.f64);
         for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
-            int tx = t % c.tile[0], r = t / c.tile[0];
-            int ty = r % c.tile[1], tz = r / c.tile[1];
+            int tx, ty, tz;
+            tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
             int s = tile_slot(c, tx, ty, tz);
             sF[3 * s] = __ldg(gF + 3 * g);
@@ -379,10 +379,10 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
 
         const LaneRange lr = lane_range(it, wid, NW);
         float vm2 = 0.f;
-        for (int64_t r = lr.first; r < lr.q; r += lr.stride) {
-            int64_t loc = lane * lr.q + r;
+        for (int r = lr.first; r < lr.q; r += lr.stride) {
+            const int loc = lane * lr.q + r;
             if (loc < lr.cnt)
-                vm2 = fmaxf(vm2, push_one_f64<D, FULL>(c, b, gm, k, lr.base + (int32_t)loc * lr.step, sF, sD, mout));
+                vm2 = fmaxf(vm2, push_one_f64<D, FULL>(c, b, gm, k, lr.base + loc * lr.step, sF, sD, mout));
         }
         unsigned vb = __reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(vm2)));
         if (lane == 0 && vb)
@@ -390,8 +390,8 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
         __syncthreads();
 
         for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
-            int tx = t % c.tile[0], r = t / c.tile[0];
-            int ty = r % c.tile[1], tz = r / c.tile[1];
+            int tx, ty, tz;
+            tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
             int s = tile_slot(c, tx, ty, tz);
             for (int ch = 0; ch < 4; ++ch) {

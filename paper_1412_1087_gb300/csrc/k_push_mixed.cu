@@ -42,6 +42,14 @@
 //    the sort's permutation by the push that applies it.  The stored
 //    four-velocity takes exactly the deposited dv (two-word sum), so the
 //    exchange with the gas conserves momentum to 2^-35 of |v| per step.
+//  * What a particle needs of its box and item sits in shared memory or
+//    registers (item_const, a lane per channel and dimension), its tile
+//    coordinate is carried along instead of found anew at each position, and
+//    the next item's number, entry, constants and field tile are fetched while
+//    the current one is pushed and flushed.  Against finding each of them when
+//    needed: two steps of 128^3 x 32 22.66 -> 21.93 ms, eight of the 1000 x 700
+//    x 64 Bell box 20.03 -> 19.47, of the shock box 9.70 -> 9.25, the coupled
+//    step of 700 x 500 x 16 678 -> 633 us.
 //  * 2-D: each thread copies its next two particles' records into a
 //    three-stage shared-memory ring with 16-byte cp.async while it pushes
 //    the current one.
@@ -80,6 +88,12 @@ struct MixedConst {
     float gs[NCH];   // global scale
     float qb[NCH];   // per-particle bound of the tile path
     int ksh[NCH];    // flush shift: global = tile * 2^ksh
+    // the box and the item as the particle loop needs them
+    int n[3];        // cells
+    int wrap[3];     // n where periodic, else 0
+    int org[3];      // box cell of tile cell 0
+    int rlo[3], rhi[3];   // tile coordinates below / above which a periodic image is nearer
+    FastDiv dnx, dnxy;
 };
 
 // TSC weights of one particle, passed by value to the global-memory path.
@@ -87,39 +101,104 @@ struct Wts {
     float x[3], y[3], z[3];
 };
 
-__device__ __forceinline__ void item_const(const BoxDev &b, float dt, int64_t cnt, int D, MixedConst &k)
+// The constants of an item, by the first 32 threads of the block: a lane per
+// channel, per dimension and for the rest (one thread computing all of them
+// kept the block waiting 2 to 3 us an item).
+__device__ __forceinline__ void item_const(const Ctx &c, const BoxDev &b, const ItemGeom &gm, float dt, int D,
+                                           MixedConst &k)
 {
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        k.hdx[d] = 0.5f * dt * (float)b.inv_dx[d];
-    float C = (float)b.C;
-    k.invC2 = 1.f / (C * C);
-    k.hh = 0.5f * (float)b.qm_cr * dt;
-    k.m = (float)b.m_cr;
-    k.qn = (float)(b.qm_cr * b.m_cr * b.inv_dV);
-    const float wmax = D == 3 ? 0.421875f : 0.5625f;   // largest TSC weight of one cell
-    // sized for the largest item, so that every item of a box has the same
-    // tile scale and a contribution rounds the same whichever item holds it
-    (void)cnt;
-    const float fc = (float)ITEM_MAX_PARTICLES + 1.f;
-    // split channels: |hi| sums <= cnt (X/2^KLO + 1) < 2^31 and |lo| sums <= cnt 2^(KLO-1) < 2^31;
-    // the hi word also needs |x| < 2^(22+KLO) for the rounding FFMA
-    const float cap_split = fminf(1099511627776.f /* 2^40 */, 524288.f * (2147483648.f / fc - 1.f));
-    // single-word channel: |x| < 2^21 and sums <= cnt x < 2^31
-    const float cap_single = fminf(2097152.f, 2147483648.f / fc);
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-        float Q = fmaxf((float)b.qbound[ch], 1e-30f);
-        int eg = b.escale[ch];
-        int et = ilogbf((ch == CH_N ? cap_single : cap_split) / (Q * wmax));   // 2^et Q wmax <= cap
+    const int l = threadIdx.x;
+    if (l < NCH) {
+        const float wmax = D == 3 ? 0.421875f : 0.5625f;   // largest TSC weight of one cell
+        // sized for the largest item, so that every item of a box has the same
+        // tile scale and a contribution rounds the same whichever item holds it
+        const float fc = (float)ITEM_MAX_PARTICLES + 1.f;
+        // split channels: |hi| sums <= cnt (X/2^KLO + 1) < 2^31 and |lo| sums <= cnt 2^(KLO-1) < 2^31;
+        // the hi word also needs |x| < 2^(22+KLO) for the rounding FFMA
+        const float cap_split = fminf(1099511627776.f /* 2^40 */, 524288.f * (2147483648.f / fc - 1.f));
+        // single-word channel: |x| < 2^21 and sums <= cnt x < 2^31
+        const float cap_single = fminf(2097152.f, 2147483648.f / fc);
+        const float Q = fmaxf((float)b.qbound[l], 1e-30f);
+        const int eg = b.escale[l];
+        int et = ilogbf((l == CH_N ? cap_single : cap_split) / (Q * wmax));   // 2^et Q wmax <= cap
         et = max(et, -SCALE_EXP_MAX);
         if (et > eg)
             et = eg;
-        k.ksh[ch] = eg - et;
-        k.st[ch] = ldexpf(1.f, et);
-        k.gs[ch] = ldexpf(1.f, eg);
-        k.qb[ch] = Q;
+        k.ksh[l] = eg - et;
+        k.st[l] = ldexpf(1.f, et);
+        k.gs[l] = ldexpf(1.f, eg);
+        k.qb[l] = Q;
+    } else if (l < NCH + 3) {
+        const int d = l - NCH;
+        const int n = b.n[d], centre = gm.half[d] + HALO;
+        const bool periodic = b.bc[d] == MHDPIC_BC_PERIODIC;
+        k.hdx[d] = 0.5f * dt * (float)b.inv_dx[d];
+        k.n[d] = n;
+        k.wrap[d] = periodic ? n : 0;
+        k.org[d] = gm.org[d];
+        k.rlo[d] = centre - n / 2;
+        k.rhi[d] = centre + n / 2;
+    } else if (l == NCH + 3) {
+        const float C = (float)b.C;
+        k.invC2 = 1.f / (C * C);
+        k.hh = 0.5f * (float)b.qm_cr * dt;
+        k.m = (float)b.m_cr;
+    } else if (l == NCH + 4) {
+        k.qn = (float)(b.qm_cr * b.m_cr * b.inv_dV);
+        k.dnx = b.div_nx;
+        k.dnxy = b.div_nxy;
     }
+}
+
+// Tile coordinate of box cell ci along d: the periodic image nearest the
+// brick's centre.
+__device__ __forceinline__ int tile_coord(const MixedConst &k, int d, int ci)
+{
+    int r = ci - k.org[d];
+    if (r > k.rhi[d])
+        r -= k.wrap[d];
+    else if (r < k.rlo[d])
+        r += k.wrap[d];
+    return r;
+}
+
+// One half-step's move along d: the offset back into [0,1), the whole cells
+// carried into the box cell ci and the tile coordinate rel, the particle
+// boundary.  A move of less than a cell within the box or across a periodic
+// face takes the short way; the others (walls, fast movers, NaN) go through
+// renorm_mixed.  True when the particle leaves the box.
+__device__ __forceinline__ bool move_mixed(const Ctx &c, const BoxDev &b, const MixedConst &k, int d, float &o, int &ci,
+                                           int &rel, float &vd)
+{
+    const bool below = o < 0.f, above = o >= 1.f;
+    int kk = above ? 1 : (below ? -1 : 0);
+    float on = above ? o - 1.f : (below ? o + 1.f : o);
+    if (on >= 1.f) {   // o was a tiny negative number that rounded up
+        on -= 1.f;
+        kk += 1;
+    }
+    int cn = ci + kk;
+    const int n = k.n[d];
+    bool odd = !(o >= -1.f && o < 2.f);
+    if ((unsigned)cn >= (unsigned)n) {
+        odd |= k.wrap[d] == 0;
+        cn = cn < 0 ? cn + n : cn - n;
+    }
+    if (odd) {
+        const bool leaving = renorm_mixed(b, d, ci, o, vd, c.status);
+        rel = tile_coord(k, d, ci);
+        return leaving;
+    }
+    o = on;
+    ci = cn;
+    rel += kk;
+    return false;
+}
+
+// The whole 3-point stencil of tile coordinate rel is inside the tile.
+__device__ __forceinline__ bool in_tile_1d(const Ctx &c, int d, int rel)
+{
+    return (unsigned)(rel - 1) <= (unsigned)(c.tile[d] - 3);
 }
 
 template <int D>
@@ -397,10 +476,24 @@ __device__ __forceinline__ void cp_async_wait_prev()
 
 // Start the copy of source particle i's two records into one stage of this
 // thread's ring (records PUSH_THREADS int4 apart).
-__device__ __forceinline__ void stage_particle(const Ctx &c, int64_t i, int4 *dst)
+__device__ __forceinline__ void stage_particle(const Ctx &c, int i, int4 *dst)
 {
     cp_async16(dst, c.src_pos + i);
     cp_async16(dst + PUSH_THREADS, c.src_vel + i);
+}
+
+// Box coordinates of a linear cell with the item's constants (decode_cell).
+template <int D>
+__device__ __forceinline__ void decode_item_cell(const MixedConst &k, int32_t cell, int ci[3])
+{
+    uint32_t r = (uint32_t)cell;
+    ci[2] = 0;
+    if (D == 3) {
+        ci[2] = (int)fdiv(r, k.dnxy);
+        r -= (uint32_t)ci[2] * k.dnxy.d;
+    }
+    ci[1] = (int)fdiv(r, k.dnx);
+    ci[0] = (int)(r - (uint32_t)ci[1] * k.dnx.d);
 }
 
 struct PIn {
@@ -430,12 +523,12 @@ __device__ __forceinline__ PIn load_staged(const int4 *in)
                                  __int_as_float(bi.w)));
 }
 
-__device__ __forceinline__ PIn load_global(const Ctx &c, int64_t i)
+__device__ __forceinline__ PIn load_global(const Ctx &c, int i)
 {
     return unpack(__ldg(c.src_pos + i), __ldg(c.src_vel + i));
 }
 
-__device__ __forceinline__ void store_particle(const Ctx &c, int64_t j, int32_t cell, const float o[3],
+__device__ __forceinline__ void store_particle(const Ctx &c, int j, int32_t cell, const float o[3],
                                                const float v[3], uint32_t res)
 {
     c.pos[j] = make_int4(cell, __float_as_int(o[0]), __float_as_int(o[1]), __float_as_int(o[2]));
@@ -460,33 +553,31 @@ __host__ __device__ inline PushLayout push_layout(int slots, int fslots)
     return l;
 }
 
-__device__ __forceinline__ void store_dead(const Ctx &c, int64_t j)
+__device__ __forceinline__ void store_dead(const Ctx &c, int j)
 {
     c.pos[j] = make_int4(DEAD_CELL, 0, 0, 0);
     c.vel[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Charge and current density deposit of one particle (eq:nJCR) at cell ci,
-// offsets o, four-velocity v with ig = 1/gamma from rsqrtf(fmaf(vsq3(v),
+// Charge and current density deposit of one particle (eq:nJCR) at box cell ci
+// and tile cell rel2, offsets o, four-velocity v with ig = 1/gamma from rsqrtf(fmaf(vsq3(v),
 // invC2, 1)): n = qn W, J = qn (v/gamma) W.  The push calls it at x^(n+1) and
 // the standalone deposit at the stored positions, so the two give the same
 // integers for the same particle state.
 template <int D>
-__device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &b, const ItemGeom &gm,
-                                                    const MixedConst &k, const int ci[3], const float o[3],
+__device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &b, const MixedConst &k,
+                                                    const int ci[3], const int rel2[3], const float o[3],
                                                     const float v[3], float ig, int *sD, unsigned long long *mout)
 {
     Wts w2;
     w2.z[0] = 0.f;
     w2.z[1] = 1.f;
     w2.z[2] = 0.f;
-    int rel2[3] = {0, 0, 0};
-    bool in2 = tile_rel(c, b, gm, 0, ci[0], rel2[0]);
-    in2 &= tile_rel(c, b, gm, 1, ci[1], rel2[1]);
+    bool in2 = in_tile_1d(c, 0, rel2[0]) && in_tile_1d(c, 1, rel2[1]);
     tsc_from_offset<float>(o[0], w2.x);
     tsc_from_offset<float>(o[1], w2.y);
     if (D == 3) {
-        in2 &= tile_rel(c, b, gm, 2, ci[2], rel2[2]);
+        in2 &= in_tile_1d(c, 2, rel2[2]);
         tsc_from_offset<float>(o[2], w2.z);
     }
     pin_weights(w2);
@@ -509,16 +600,18 @@ __device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &
 }
 
 template <int D, bool FULL>
-__device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const ItemGeom &gm, const MixedConst &k,
-                                          int64_t j, const PIn &pin, const float4 *sFa, const float2 *sFb,
-                                          int *sD, unsigned long long *mout)
+__device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const MixedConst &k, int j, const PIn &pin,
+                                          const float4 *sFa, const float2 *sFb, int *sD, unsigned long long *mout)
 {
     if (pin.cell == DEAD_CELL) {   // left the box earlier (kept until the next sort)
         store_dead(c, j);
         return 0.f;
     }
-    int ci[3];
-    decode_cell(b, pin.cell, ci);
+    int ci[3], rel[3] = {0, 0, 0};
+    decode_item_cell<D>(k, pin.cell, ci);
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+        rel[d] = tile_coord(k, d, ci[d]);
     float o[3] = {pin.o[0], pin.o[1], pin.o[2]}, v[3] = {pin.v[0], pin.v[1], pin.v[2]};
 
     // drift to x^(n+1/2) with u = v / gamma (a particle at an open face is
@@ -529,20 +622,18 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const I
 #pragma unroll
     for (int d = 0; d < D; ++d) {
         o[d] = fmaf(k.hdx[d] * ign, v[d], o[d]);
-        leaving |= renorm_mixed(b, d, ci[d], o[d], v[d], c.status);
+        leaving |= move_mixed(c, b, k, d, o[d], ci[d], rel[d], v[d]);
     }
 
     Wts w;
     w.z[0] = 0.f;
     w.z[1] = 1.f;
     w.z[2] = 0.f;
-    int rel[3] = {0, 0, 0};
-    bool in_tile = tile_rel(c, b, gm, 0, ci[0], rel[0]);
-    in_tile &= tile_rel(c, b, gm, 1, ci[1], rel[1]);
+    bool in_tile = in_tile_1d(c, 0, rel[0]) && in_tile_1d(c, 1, rel[1]);
     tsc_from_offset<float>(o[0], w.x);
     tsc_from_offset<float>(o[1], w.y);
     if (D == 3) {
-        in_tile &= tile_rel(c, b, gm, 2, ci[2], rel[2]);
+        in_tile &= in_tile_1d(c, 2, rel[2]);
         tsc_from_offset<float>(o[2], w.z);
     }
     pin_weights(w);
@@ -630,7 +721,7 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const I
     for (int d = 0; d < D; ++d) {
         o[d] = fmaf(k.hdx[d] * ig2, vn[d], o[d]);
         const float before = vn[d];
-        leaving |= renorm_mixed(b, d, ci[d], o[d], vn[d], c.status);
+        leaving |= move_mixed(c, b, k, d, o[d], ci[d], rel[d], vn[d]);
         if (vn[d] != before)
             rq[d] = -rq[d];
     }
@@ -641,11 +732,12 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const I
     }
 
     if (FULL)
-        deposit_moments_one<D>(c, b, gm, k, ci, o, vn, ig2, sD, mout);
+        deposit_moments_one<D>(c, b, k, ci, rel, o, vn, ig2, sD, mout);
 
     if (!isfinite(vn[0] + vn[1] + vn[2]))
         set_status(c.status, MHDPIC_ST_NONFINITE);
-    store_particle(c, j, (int32_t)(((int64_t)ci[2] * b.n[1] + ci[1]) * b.n[0] + ci[0]), o, vn, res_pack(rq));
+    const int row = D == 3 ? ci[2] * k.n[1] + ci[1] : ci[1];
+    store_particle(c, j, row * k.n[0] + ci[0], o, vn, res_pack(rq));
     return vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2];
 }
 
@@ -696,52 +788,65 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
             mbar_init(&s_bar);
         __syncthreads();
     }
-    __shared__ int s_item;
-    __shared__ MixedConst s_k;
+    // the work item at hand and the next: the next one's number, entry and
+    // constants are fetched while this one is pushed and flushed
+    __shared__ WorkItem s_it[2];
+    __shared__ MixedConst s_k[2];
+    __shared__ int s_item[2];
     unsigned long long *mout = c.momdep[cur_out];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int NW = PUSH_THREADS / 32;
 
-    for (;;) {
-        if (threadIdx.x == 0)
-            s_item = atomicAdd(work_ctr, 1);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= nit)
-            break;
-        const WorkItem it = items[item];
-        const BoxDev &b = c.boxes[it.box];
-        const ItemGeom gm = item_geom(c, b, it.brick, D);
-
-        // stage the fields: the tile is one block of the padded planes
-        // (ghosts included), copied by the tensor engine or by the threads
-        if (c.tma) {
-            if (threadIdx.x == 0) {
-                // the previous item's reads of the tile ended at the barrier before
-                fence_proxy_async();
-                mbar_expect_tx(&s_bar, copy_bytes);
-                const unsigned char *tm = c.tmaps + (size_t)it.box * 256;
-                const int x0 = gm.org[0] + FGHOST, y0 = gm.org[1] + FGHOST, z0 = gm.org[2] + FGHOST;
-                tma_tile<D>(sFa, tm, 4 * x0, y0, z0, &s_bar);
-                tma_tile<D>(sFb, tm + 128, 2 * x0, y0, z0, &s_bar);
-            }
-        } else {
-            for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
-                const int tx = t % c.tile[0], r = t / c.tile[0];
-                const int ty = r % c.tile[1], tz = r / c.tile[1];
-                // the tile lies inside the padded planes (they cover the brick grid plus the halo)
-                const int64_t f = fidx(b, gm.org[0] + tx, gm.org[1] + ty, gm.org[2] + tz);
-                const int sl = tx + c.fts[1] * ty + c.fts[2] * tz;
-                sFa[sl] = __ldg(c.fa + f);
-                sFb[sl] = __ldg(c.fb + f);
-            }
+    // the fields of an item: the tile is one block of the padded planes
+    // (ghosts included), copied by the tensor engine or by the threads
+    auto copy_fields = [&](const WorkItem &it, const MixedConst &k) {   // one thread
+        fence_proxy_async();   // the last reads of the tile ended at a barrier before
+        mbar_expect_tx(&s_bar, copy_bytes);
+        const unsigned char *tm = c.tmaps + (size_t)it.box * 256;
+        const int x0 = k.org[0] + FGHOST, y0 = k.org[1] + FGHOST, z0 = k.org[2] + FGHOST;
+        tma_tile<D>(sFa, tm, 4 * x0, y0, z0, &s_bar);
+        tma_tile<D>(sFb, tm + 128, 2 * x0, y0, z0, &s_bar);
+    };
+    // warp 0: the entry and the constants of item number `item` into buffer q
+    auto fetch_item = [&](int item, int q) {
+        if (lane == 0)
+            s_item[q] = item;
+        if (item < nit) {
+            const WorkItem it = items[item];
+            const BoxDev &b = c.boxes[it.box];
+            item_const(c, b, item_geom(c, b, it.brick, D), dt, D, s_k[q]);
+            if (lane == 0)
+                s_it[q] = it;
         }
-        // clear the deposit tile and its counts
-        for (int s = threadIdx.x; s < TILE_WORDS * S; s += PUSH_THREADS)
-            sD[s] = 0;
+    };
+    // clear the deposit tile and its counts (whole 16-byte words: the tile's
+    // part of the shared memory is a multiple of 128 bytes)
+    auto clear_tile = [&] {
+        int4 *z = reinterpret_cast<int4 *>(sD);
+        for (int s = threadIdx.x; s < (TILE_WORDS * S + 3) / 4; s += PUSH_THREADS)
+            z[s] = make_int4(0, 0, 0, 0);
+    };
+
+    if (wid == 0) {
+        int first = 0;
+        if (lane == 0)
+            first = atomicAdd(work_ctr, 1);
+        fetch_item(__shfl_sync(0xffffffffu, first, 0), 0);
+        __syncwarp();
+        if (c.tma && lane == 0 && s_item[0] < nit)
+            copy_fields(s_it[0], s_k[0]);
+    }
+    clear_tile();
+    __syncthreads();
+
+    for (int q = 0;; q ^= 1) {
+        if (s_item[q] >= nit)
+            break;
+        const WorkItem it = s_it[q];
+        const BoxDev &b = c.boxes[it.box];
+        int next = 0;
         if (threadIdx.x == 0)
-            item_const(b, dt, it.p1 - it.p0, D, s_k);
-        __syncthreads();
+            next = atomicAdd(work_ctr, 1);   // used after the particles
         if (c.tma) {
             const bool ok = mbar_wait(&s_bar, phase, c.copy_limit_ns);
             if (__syncthreads_or(!ok)) {   // give up the launch, after the copies in flight have had their time
@@ -751,28 +856,38 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
                 return;
             }
             phase ^= 1u;
+        } else {
+            const MixedConst &k = s_k[q];
+            for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
+                int tx, ty, tz;
+                tile_cell(c, t, tx, ty, tz);
+                // the tile lies inside the padded planes (they cover the brick grid plus the halo)
+                const int64_t f = fidx(b, k.org[0] + tx, k.org[1] + ty, k.org[2] + tz);
+                const int sl = tx + c.fts[1] * ty + c.fts[2] * tz;
+                sFa[sl] = __ldg(c.fa + f);
+                sFb[sl] = __ldg(c.fb + f);
+            }
+            __syncthreads();
         }
         // the item constants stay in shared memory where registers are short
         MixedConst kreg;
         if (!CONST_IN_SMEM<D>)
-            kreg = s_k;
-        const MixedConst &k = CONST_IN_SMEM<D> ? s_k : kreg;
+            kreg = s_k[q];
+        const MixedConst &k = CONST_IN_SMEM<D> ? s_k[q] : kreg;
 
         float vm2 = 0.f;
         {
             const LaneRange lr = lane_range(it, wid, NW);
-            const int64_t base = lr.base, cnt = lr.cnt, lane0 = lane * lr.q, rb = lr.first, re = lr.q,
-                          rs = lr.stride;
-            const int32_t step = lr.step;
+            const int lane0 = lane * lr.q, re = min(lr.q, lr.cnt - lane0), rs = lr.stride;   // this lane's rounds end at re
             // source particle of sorted position base + (lane0 + r) step; when the
             // push applies a sort the permutation entry is loaded one
             // iteration early.  (One code path for both cases, so that the
             // arithmetic is the same instruction for instruction.)
             const bool gather = c.perm_src != nullptr;
-            auto valid = [&](int64_t r) { return r < re && lane0 + r < cnt; };
-            auto src_of = [&](int64_t r) -> int64_t {
-                const int64_t j = base + (int32_t)(lane0 + r) * step;
-                return gather ? (int64_t)__ldg(c.perm_src + j) : j;
+            const int base = lr.base + lane0 * lr.step;
+            auto src_of = [&](int r) {
+                const int j = base + r * lr.step;
+                return gather ? __ldg(c.perm_src + j) : j;
             };
             if (STAGED<D>) {
                 // the next RING_STAGES - 1 particles' words are copied into
@@ -780,47 +895,52 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
                 constexpr int NS = RING_STAGES;
 #pragma unroll
                 for (int s0 = 0; s0 < NS - 1; ++s0) {
-                    if (valid(rb + s0 * rs))
-                        stage_particle(c, src_of(rb + s0 * rs), ring + s0 * RS);
+                    if (lr.first + s0 * rs < re)
+                        stage_particle(c, src_of(lr.first + s0 * rs), ring + s0 * RS);
                     cp_async_commit();
                 }
-                int64_t sn = valid(rb + (NS - 1) * rs) ? src_of(rb + (NS - 1) * rs) : 0;
+                int sn = lr.first + (NS - 1) * rs < re ? src_of(lr.first + (NS - 1) * rs) : 0;
                 int st = 0;
-                for (int64_t r = rb; r < re; r += rs) {
+                for (int r = lr.first; r < lr.q; r += rs) {
                     const int stn = st == 0 ? NS - 1 : st - 1;
-                    if (valid(r + (NS - 1) * rs))
+                    if (r + (NS - 1) * rs < re)
                         stage_particle(c, sn, ring + stn * RS);
-                    if (valid(r + NS * rs))
+                    if (r + NS * rs < re)
                         sn = src_of(r + NS * rs);
                     cp_async_commit();
                     cp_async_wait_prev();
-                    if (lane0 + r < cnt)
-                        vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, gm, k, base + (int32_t)(lane0 + r) * step, load_staged(ring + st * RS),
+                    if (r < re)
+                        vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, k, base + r * lr.step, load_staged(ring + st * RS),
                                                            sFa, sFb, sD, mout));
                     st = st + 1 == NS ? 0 : st + 1;
                 }
             } else {
-                int64_t sn = valid(rb) ? src_of(rb) : 0;
-                for (int64_t r = rb; r < re; r += rs)
-                    if (lane0 + r < cnt) {
-                        const int64_t src = sn;
-                        if (valid(r + rs))
-                            sn = src_of(r + rs);
-                        vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, gm, k, base + (int32_t)(lane0 + r) * step, load_global(c, src), sFa,
-                                                           sFb, sD, mout));
-                    }
+                int sn = lr.first < re ? src_of(lr.first) : 0;
+                for (int r = lr.first; r < re; r += rs) {
+                    const int src = sn;
+                    if (r + rs < re)
+                        sn = src_of(r + rs);
+                    vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, k, base + r * lr.step, load_global(c, src), sFa, sFb, sD,
+                                                       mout));
+                }
             }
         }
         unsigned vb = __reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(vm2)));
         if (lane == 0 && vb)
             atomicMax(&c.stats[it.box].vmax, vb);
+        if (wid == 0)
+            fetch_item(__shfl_sync(0xffffffffu, next, 0), q ^ 1);
         __syncthreads();
+        // the fields of the next item land while this one is flushed
+        if (c.tma && threadIdx.x == 0 && s_item[q ^ 1] < nit)
+            copy_fields(s_it[q ^ 1], s_k[q ^ 1]);
 
         // remove the offsets, rebuild hi 2^KLO + lo and shift the tile into
         // the global accumulators
+        const ItemGeom gm = item_geom(c, b, it.brick, D);
         for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
-            int tx = t % c.tile[0], r = t / c.tile[0];
-            int ty = r % c.tile[1], tz = r / c.tile[1];
+            int tx, ty, tz;
+            tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
             int s = tile_slot(c, tx, ty, tz);
             const uint32_t kc = slot_count(c, sD, W_CNT_C, tx, ty, tz, D);
@@ -832,10 +952,12 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
                 const long long v = slot_value(sD, s, ch, kc, km);
                 if (v) {
                     unsigned long long *dst = ch < CH_N ? c.corr + ch * c.nc + g : mout + (ch - CH_N) * c.nc + g;
-                    atomicAdd(dst, (unsigned long long)v << k.ksh[ch]);
+                    atomicAdd(dst, (unsigned long long)v << s_k[q].ksh[ch]);
                 }
             }
         }
+        __syncthreads();
+        clear_tile();
         __syncthreads();
     }
 }
@@ -956,31 +1078,33 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_deposit_mixed(Ctx c, const Wor
         const ItemGeom gm = item_geom(c, b, it.brick, D);
         for (int s = threadIdx.x; s < TILE_WORDS * S; s += PUSH_THREADS)
             sD[s] = 0;
-        if (threadIdx.x == 0)
-            item_const(b, 0.f, it.p1 - it.p0, D, s_k);
+        if (threadIdx.x < 32)
+            item_const(c, b, gm, 0.f, D, s_k);
         __syncthreads();
         const MixedConst &k = s_k;
         {
             const LaneRange lr = lane_range(it, wid, NW);
-            const int64_t lane0 = lane * lr.q;
-            for (int64_t r = lr.first; r < lr.q; r += lr.stride) {
+            const int lane0 = lane * lr.q;
+            for (int r = lr.first; r < lr.q; r += lr.stride) {
                 if (lane0 + r >= lr.cnt)
                     continue;
-                const int64_t j = lr.base + (int32_t)(lane0 + r) * lr.step;
-                const int64_t src = gather ? (int64_t)__ldg(c.perm_src + j) : j;
-                const PIn pin = load_global(c, src);
+                const int j = lr.base + (lane0 + r) * lr.step;
+                const PIn pin = load_global(c, gather ? __ldg(c.perm_src + j) : j);
                 if (pin.cell == DEAD_CELL)
                     continue;
-                int ci[3];
-                decode_cell(b, pin.cell, ci);
+                int ci[3], rel[3] = {0, 0, 0};
+                decode_item_cell<D>(k, pin.cell, ci);
+#pragma unroll
+                for (int d = 0; d < D; ++d)
+                    rel[d] = tile_coord(k, d, ci[d]);
                 const float ig = rsqrtf(fmaf(vsq3(pin.v), k.invC2, 1.f));
-                deposit_moments_one<D>(c, b, gm, k, ci, pin.o, pin.v, ig, sD, mout);
+                deposit_moments_one<D>(c, b, k, ci, rel, pin.o, pin.v, ig, sD, mout);
             }
         }
         __syncthreads();
         for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
-            int tx = t % c.tile[0], r = t / c.tile[0];
-            int ty = r % c.tile[1], tz = r / c.tile[1];
+            int tx, ty, tz;
+            tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
             int s = tile_slot(c, tx, ty, tz);
             const uint32_t km = slot_count(c, sD, W_CNT_M, tx, ty, tz, D);

@@ -652,6 +652,8 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
                 k.brick_sh[d] = sh;
     }
     k.tile_vol = k.tile[0] * k.tile[1] * k.tile[2];
+    k.tdx = make_fastdiv((uint32_t)k.tile[0]);
+    k.tdxy = make_fastdiv((uint32_t)(k.tile[0] * k.tile[1]));
     // Default 64-cell bricks are worked as two 32-cell halves, one lane per
     // cell; the tile strides are padded so those 32 cells hit 32 banks.
     k.halves = 0;

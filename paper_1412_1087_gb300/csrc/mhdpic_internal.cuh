@@ -123,6 +123,7 @@ struct Ctx {
     int32_t brick_sh[3];   // log2 of brick[d] when it is a power of two, else -1
     int32_t tile[3];       // brick + 2*HALO
     int32_t tile_vol;      // cells of the tile
+    FastDiv tdx, tdxy;     // division by tile[0] and tile[0] tile[1]
     int32_t ts[3];         // tile strides in slots (x, y, z); padded to spread banks
     int32_t tile_slots;    // slots of the tile (>= tile_vol)
     int32_t fts[3];        // field tile strides (x 1, y ts[1], z dense): the layout a tensor copy writes

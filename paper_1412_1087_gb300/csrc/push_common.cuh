@@ -188,12 +188,10 @@ __device__ __forceinline__ void stencil_coords(const BoxDev &b, const int ci[3],
 // Split of an item's particles over the block's warps: with halves, warps
 // 0..NW/2-1 take [p0, pm) and the rest [pm, p1); lane l works through the
 // l-th 1/32 of its range, the warps of a group interleaving inside it.  The
-// range's k-th particle sits at position base + k * step (k * step stays
-// below 2^31: an item holds at most ITEM_MAX_PARTICLES).
+// range's k-th particle sits at position base + k * step (positions are below
+// 2^31, and so is the number of particles).
 struct LaneRange {
-    int64_t base, cnt, q;
-    int32_t step;
-    int first, stride;
+    int32_t base, cnt, q, step, first, stride;
 };
 
 __device__ __forceinline__ LaneRange lane_range(const WorkItem &it, int wid, int nw)
@@ -202,13 +200,13 @@ __device__ __forceinline__ LaneRange lane_range(const WorkItem &it, int wid, int
     if (it.pm >= 0) {
         int half = nw / 2;
         bool hi = wid >= half;
-        r.base = hi ? it.pm : it.p0;
-        r.cnt = hi ? it.p1 - it.pm : it.pm - it.p0;
+        r.base = (int32_t)(hi ? it.pm : it.p0);
+        r.cnt = (int32_t)(hi ? it.p1 - it.pm : it.pm - it.p0);
         r.first = hi ? wid - half : wid;
         r.stride = half;
         r.step = 1;
     } else {
-        r.base = it.p0;
+        r.base = (int32_t)it.p0;
         r.step = it.step;
         r.cnt = it.count;
         r.first = wid;
@@ -216,6 +214,15 @@ __device__ __forceinline__ LaneRange lane_range(const WorkItem &it, int wid, int
     }
     r.q = (r.cnt + 31) / 32;
     return r;
+}
+
+// Coordinates of tile cell t (x fastest).
+__device__ __forceinline__ void tile_cell(const Ctx &c, int t, int &tx, int &ty, int &tz)
+{
+    tz = (int)fdiv((uint32_t)t, c.tdxy);
+    const int r = t - tz * (int)c.tdxy.d;
+    ty = (int)fdiv((uint32_t)r, c.tdx);
+    tx = r - ty * (int)c.tdx.d;
 }
 
 }  // namespace mhdpic

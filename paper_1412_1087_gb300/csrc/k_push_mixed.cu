@@ -50,9 +50,8 @@
 //    needed: two steps of 128^3 x 32 22.66 -> 21.93 ms, eight of the 1000 x 700
 //    x 64 Bell box 20.03 -> 19.47, of the shock box 9.70 -> 9.25, the coupled
 //    step of 700 x 500 x 16 678 -> 633 us.
-//  * 2-D: each thread copies its next two particles' records into a
-//    three-stage shared-memory ring with 16-byte cp.async while it pushes
-//    the current one.
+//  * 2-D: each thread copies its next particle's records into a two-stage
+//    shared-memory ring with 16-byte cp.async while it pushes the current one.
 #include "async_copy.cuh"
 #include "cells_common.cuh"
 #include "push_common.cuh"
@@ -78,22 +77,27 @@ constexpr int W_LO = NCH;               // lo word of channel ch: W_LO + ch
 constexpr int W_CNT_M = NCH + CH_N;     // contributions of the moments deposit, by stencil corner
 constexpr int W_CNT_C = 2 * NCH;        // the same for the corrector deposit
 
-struct MixedConst {
+// What every particle of an item needs of its box: kept in registers where
+// there are enough.
+struct HotConst {
     float hdx[3];    // dt / (2 dx)
     float invC2;     // 1 / C^2
     float hh;        // (q/mc) dt / 2
     float m;
     float qn;        // (q/mc) m / dV
     float st[NCH];   // tile scale
-    float gs[NCH];   // global scale
     float qb[NCH];   // per-particle bound of the tile path
+};
+
+// An item's constants, in shared memory.  The integers are read four at a time.
+struct MixedConst {
+    HotConst h;
+    float gs[NCH];   // global scale
     int ksh[NCH];    // flush shift: global = tile * 2^ksh
-    // the box and the item as the particle loop needs them
-    int n[3];        // cells
-    int wrap[3];     // n where periodic, else 0
-    int org[3];      // box cell of tile cell 0
-    int rlo[3], rhi[3];   // tile coordinates below / above which a periodic image is nearer
-    FastDiv dnx, dnxy;
+    int4 dim[3];     // box cell of tile cell 0; tile coordinates below and above which a periodic image is
+                     // nearer; cells where periodic, else 0
+    int4 n;          // cells of the box, and of its x y plane
+    int4 div;        // the divisions by n.x and n.w (FastDiv mul, shift)
 };
 
 // TSC weights of one particle, passed by value to the global-memory path.
@@ -125,49 +129,44 @@ __device__ __forceinline__ void item_const(const Ctx &c, const BoxDev &b, const 
         if (et > eg)
             et = eg;
         k.ksh[l] = eg - et;
-        k.st[l] = ldexpf(1.f, et);
+        k.h.st[l] = ldexpf(1.f, et);
         k.gs[l] = ldexpf(1.f, eg);
-        k.qb[l] = Q;
+        k.h.qb[l] = Q;
     } else if (l < NCH + 3) {
         const int d = l - NCH;
         const int n = b.n[d], centre = gm.half[d] + HALO;
-        const bool periodic = b.bc[d] == MHDPIC_BC_PERIODIC;
-        k.hdx[d] = 0.5f * dt * (float)b.inv_dx[d];
-        k.n[d] = n;
-        k.wrap[d] = periodic ? n : 0;
-        k.org[d] = gm.org[d];
-        k.rlo[d] = centre - n / 2;
-        k.rhi[d] = centre + n / 2;
+        k.h.hdx[d] = 0.5f * dt * (float)b.inv_dx[d];
+        k.dim[d] = make_int4(gm.org[d], centre - n / 2, centre + n / 2, b.bc[d] == MHDPIC_BC_PERIODIC ? n : 0);
     } else if (l == NCH + 3) {
         const float C = (float)b.C;
-        k.invC2 = 1.f / (C * C);
-        k.hh = 0.5f * (float)b.qm_cr * dt;
-        k.m = (float)b.m_cr;
+        k.h.invC2 = 1.f / (C * C);
+        k.h.hh = 0.5f * (float)b.qm_cr * dt;
+        k.h.m = (float)b.m_cr;
     } else if (l == NCH + 4) {
-        k.qn = (float)(b.qm_cr * b.m_cr * b.inv_dV);
-        k.dnx = b.div_nx;
-        k.dnxy = b.div_nxy;
+        k.h.qn = (float)(b.qm_cr * b.m_cr * b.inv_dV);
+        k.n = make_int4(b.n[0], b.n[1], b.n[2], (int)b.div_nxy.d);
+        k.div = make_int4((int)b.div_nx.mul, (int)b.div_nx.shift, (int)b.div_nxy.mul, (int)b.div_nxy.shift);
     }
 }
 
-// Tile coordinate of box cell ci along d: the periodic image nearest the
-// brick's centre.
-__device__ __forceinline__ int tile_coord(const MixedConst &k, int d, int ci)
+// Tile coordinate of box cell ci along a dimension (MixedConst::dim): the
+// periodic image nearest the brick's centre.
+__device__ __forceinline__ int tile_coord(const int4 m, int ci)
 {
-    int r = ci - k.org[d];
-    if (r > k.rhi[d])
-        r -= k.wrap[d];
-    else if (r < k.rlo[d])
-        r += k.wrap[d];
+    int r = ci - m.x;
+    if (r > m.z)
+        r -= m.w;
+    else if (r < m.y)
+        r += m.w;
     return r;
 }
 
 // One half-step's move along d: the offset back into [0,1), the whole cells
-// carried into the box cell ci and the tile coordinate rel, the particle
-// boundary.  A move of less than a cell within the box or across a periodic
-// face takes the short way; the others (walls, fast movers, NaN) go through
-// renorm_mixed.  True when the particle leaves the box.
-__device__ __forceinline__ bool move_mixed(const Ctx &c, const BoxDev &b, const MixedConst &k, int d, float &o, int &ci,
+// carried into the box cell ci (of n) and the tile coordinate rel, the
+// particle boundary.  A move of less than a cell within the box or across a
+// periodic face takes the short way; the others (walls, fast movers, NaN) go
+// through renorm_mixed.  True when the particle leaves the box.
+__device__ __forceinline__ bool move_mixed(const Ctx &c, const BoxDev &b, const int4 m, int n, int d, float &o, int &ci,
                                            int &rel, float &vd)
 {
     const bool below = o < 0.f, above = o >= 1.f;
@@ -178,15 +177,14 @@ __device__ __forceinline__ bool move_mixed(const Ctx &c, const BoxDev &b, const 
         kk += 1;
     }
     int cn = ci + kk;
-    const int n = k.n[d];
     bool odd = !(o >= -1.f && o < 2.f);
     if ((unsigned)cn >= (unsigned)n) {
-        odd |= k.wrap[d] == 0;
+        odd |= m.w == 0;
         cn = cn < 0 ? cn + n : cn - n;
     }
     if (odd) {
         const bool leaving = renorm_mixed(b, d, ci, o, vd, c.status);
-        rel = tile_coord(k, d, ci);
+        rel = tile_coord(m, ci);
         return leaving;
     }
     o = on;
@@ -443,20 +441,21 @@ __device__ __forceinline__ bool within(const float q[4], const float *qb, int ch
 
 // Particle records staged per thread: pos and vel, 16 bytes each.
 constexpr int RING_RECS = 2;
-constexpr int RING_STAGES = 3;
+constexpr int RING_STAGES = 2;
 // Per dimension: 2-D pushes are short, so the kernel hides the particle
-// loads behind a three-stage shared-memory ring (two particles ahead) and
-// runs 3 CTAs per SM (80 registers, no
-// spills in the loop; 4 CTAs at 64 registers spilled and measured slower with
-// a sort every step) with the item constants in shared memory; 3-D pushes
-// keep everything in registers at 2 CTAs per SM (the ring measured no faster
-// there and takes shared memory from L1).
+// loads behind a two-stage shared-memory ring (one particle ahead; three
+// stages 1% slower since the loop's integer work went) and runs 3 CTAs per SM
+// (80 registers; 4 CTAs at 64 registers measured 10% slower) with the item's
+// integers read from shared memory; 3-D pushes, whose bound is the shared
+// memory pipe, keep them and the next particle's records in registers at 2
+// CTAs per SM (two steps of 128^3 x 32: 22.0 ms with the records loaded when
+// needed, 22.3 with the integers in shared memory, 21.7 so).
 template <int D>
 constexpr bool STAGED = D == 2;
 template <int D>
 constexpr int MIN_BLOCKS = D == 3 ? 2 : 3;
 template <int D>
-constexpr bool CONST_IN_SMEM = D == 2;
+constexpr bool INTS_IN_SMEM = D == 2;
 
 __device__ __forceinline__ void cp_async16(int4 *dst, const void *src)
 {
@@ -484,16 +483,16 @@ __device__ __forceinline__ void stage_particle(const Ctx &c, int i, int4 *dst)
 
 // Box coordinates of a linear cell with the item's constants (decode_cell).
 template <int D>
-__device__ __forceinline__ void decode_item_cell(const MixedConst &k, int32_t cell, int ci[3])
+__device__ __forceinline__ void decode_item_cell(const int4 n, const int4 div, int32_t cell, int ci[3])
 {
     uint32_t r = (uint32_t)cell;
     ci[2] = 0;
     if (D == 3) {
-        ci[2] = (int)fdiv(r, k.dnxy);
-        r -= (uint32_t)ci[2] * k.dnxy.d;
+        ci[2] = (int)((__umulhi(r, (uint32_t)div.z) + r) >> div.w);
+        r -= (uint32_t)(ci[2] * n.w);
     }
-    ci[1] = (int)fdiv(r, k.dnx);
-    ci[0] = (int)(r - (uint32_t)ci[1] * k.dnx.d);
+    ci[1] = (int)((__umulhi(r, (uint32_t)div.x) + r) >> div.y);
+    ci[0] = (int)(r - (uint32_t)(ci[1] * n.x));
 }
 
 struct PIn {
@@ -565,8 +564,8 @@ __device__ __forceinline__ void store_dead(const Ctx &c, int j)
 // the standalone deposit at the stored positions, so the two give the same
 // integers for the same particle state.
 template <int D>
-__device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &b, const MixedConst &k,
-                                                    const int ci[3], const int rel2[3], const float o[3],
+__device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &b, const HotConst &h,
+                                                    const MixedConst &k, const int ci[3], const int rel2[3], const float o[3],
                                                     const float v[3], float ig, int *sD, unsigned long long *mout)
 {
     Wts w2;
@@ -581,11 +580,11 @@ __device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &
         tsc_from_offset<float>(o[2], w2.z);
     }
     pin_weights(w2);
-    const float qj = k.qn * ig;
-    const float qm[4] = {pinned(k.qn), pinned(qj * v[0]), pinned(qj * v[1]), pinned(qj * v[2])};
-    if (within(qm, k.qb, CH_N)) {
-        const float qs[4] = {pinned(qm[0] * k.st[4]), pinned(qm[1] * k.st[5]), pinned(qm[2] * k.st[6]),
-                             pinned(qm[3] * k.st[7])};
+    const float qj = h.qn * ig;
+    const float qm[4] = {pinned(h.qn), pinned(qj * v[0]), pinned(qj * v[1]), pinned(qj * v[2])};
+    if (within(qm, h.qb, CH_N)) {
+        const float qs[4] = {pinned(qm[0] * h.st[4]), pinned(qm[1] * h.st[5]), pinned(qm[2] * h.st[6]),
+                             pinned(qm[3] * h.st[7])};
         if (in2) {
             const int base2 = (rel2[0] - 1) + c.ts[1] * (rel2[1] - 1) + (D == 3 ? c.ts[2] * (rel2[2] - 1) : 0);
             deposit_tile<D>(c, base2, w2, qs, CH_N, sD);
@@ -600,7 +599,8 @@ __device__ __forceinline__ void deposit_moments_one(const Ctx &c, const BoxDev &
 }
 
 template <int D, bool FULL>
-__device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const MixedConst &k, int j, const PIn &pin,
+__device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const HotConst &h, const MixedConst &k, int j,
+                                          const PIn &pin,
                                           const float4 *sFa, const float2 *sFb, int *sD, unsigned long long *mout)
 {
     if (pin.cell == DEAD_CELL) {   // left the box earlier (kept until the next sort)
@@ -608,21 +608,23 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const M
         return 0.f;
     }
     int ci[3], rel[3] = {0, 0, 0};
-    decode_item_cell<D>(k, pin.cell, ci);
+    const int4 n4 = k.n;
+    decode_item_cell<D>(n4, k.div, pin.cell, ci);
+    const int n[3] = {n4.x, n4.y, n4.z};
 #pragma unroll
     for (int d = 0; d < D; ++d)
-        rel[d] = tile_coord(k, d, ci[d]);
+        rel[d] = tile_coord(k.dim[d], ci[d]);
     float o[3] = {pin.o[0], pin.o[1], pin.o[2]}, v[3] = {pin.v[0], pin.v[1], pin.v[2]};
 
     // drift to x^(n+1/2) with u = v / gamma (a particle at an open face is
     // held just inside it, deposits its corrector and then leaves)
-    const float sn = fmaf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2], k.invC2, 1.f);   // gamma^2
+    const float sn = fmaf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2], h.invC2, 1.f);   // gamma^2
     const float ign = rsqrtf(sn);
     bool leaving = false;
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-        o[d] = fmaf(k.hdx[d] * ign, v[d], o[d]);
-        leaving |= move_mixed(c, b, k, d, o[d], ci[d], rel[d], v[d]);
+        o[d] = fmaf(h.hdx[d] * ign, v[d], o[d]);
+        leaving |= move_mixed(c, b, k.dim[d], n[d], d, o[d], ci[d], rel[d], v[d]);
     }
 
     Wts w;
@@ -663,11 +665,11 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const M
     }
 
     // Boris: v0 = v + (h/2)E; b = (h/2)B/gamma(v0); v1 = v0 + 2(v0 + v0 x b) x b/(1+b^2)
-    const float e0 = k.hh * E[0], e1 = k.hh * E[1], e2 = k.hh * E[2];
+    const float e0 = h.hh * E[0], e1 = h.hh * E[1], e2 = h.hh * E[2];
     const float v00 = v[0] + e0, v01 = v[1] + e1, v02 = v[2] + e2;
-    const float s1 = fmaf(v00 * v00 + v01 * v01 + v02 * v02, k.invC2, 1.f);
+    const float s1 = fmaf(v00 * v00 + v01 * v01 + v02 * v02, h.invC2, 1.f);
     const float ig1 = rsqrtf(s1);
-    const float hb = k.hh * ig1;
+    const float hb = h.hh * ig1;
     const float b0 = hb * Bf[0], b1 = hb * Bf[1], b2 = hb * Bf[2];
     const float t0 = v00 + (v01 * b2 - v02 * b1), t1 = v01 + (v02 * b0 - v00 * b2),
                 t2 = v02 + (v00 * b1 - v01 * b0);
@@ -680,17 +682,17 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const M
 
     // dv = h E + rot without cancellation; the rotation keeps |v|, so dE_k is
     // the change of the two half kicks, E_k(a) - E_k(b) = (a-b).(a+b)/(ga+gb)
-    const float s2k = fmaf(vsq3(vk), k.invC2, 1.f);
+    const float s2k = fmaf(vsq3(vk), h.invC2, 1.f);
     const float ig2k = rsqrtf(s2k);
     const float gn = sn * ign, g1 = s1 * ig1, g2 = s2k * ig2k;   // gamma = gamma^2 / gamma
     const float dEk = __fdividef(e0 * (vk[0] + v10) + e1 * (vk[1] + v11) + e2 * (vk[2] + v12), g2 + g1) +
                       __fdividef(e0 * (v00 + v[0]) + e1 * (v01 + v[1]) + e2 * (v02 + v[2]), g1 + gn);
     const float dv[3] = {pinned(2.f * e0 + r0), pinned(2.f * e1 + r1), pinned(2.f * e2 + r2)};
     {
-        const float qc[4] = {pinned(-k.m * dv[0]), pinned(-k.m * dv[1]), pinned(-k.m * dv[2]), pinned(-k.m * dEk)};
-        if (within(qc, k.qb, CH_MX)) {
-            const float qs[4] = {pinned(qc[0] * k.st[0]), pinned(qc[1] * k.st[1]), pinned(qc[2] * k.st[2]),
-                                 pinned(qc[3] * k.st[3])};
+        const float qc[4] = {pinned(-h.m * dv[0]), pinned(-h.m * dv[1]), pinned(-h.m * dv[2]), pinned(-h.m * dEk)};
+        if (within(qc, h.qb, CH_MX)) {
+            const float qs[4] = {pinned(qc[0] * h.st[0]), pinned(qc[1] * h.st[1]), pinned(qc[2] * h.st[2]),
+                                 pinned(qc[3] * h.st[3])};
             if (in_tile)
                 deposit_tile<D>(c, base, w, qs, CH_MX, sD);
             else
@@ -714,14 +716,14 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const M
 #pragma unroll
     for (int d = 0; d < 3; ++d)
         two_word_add(vn[d], rq[d], dv[d]);
-    const float ig2 = rsqrtf(fmaf(vsq3(vn), k.invC2, 1.f));
+    const float ig2 = rsqrtf(fmaf(vsq3(vn), h.invC2, 1.f));
 
     // drift to x^(n+1); a reflection mirrors both words of the component
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-        o[d] = fmaf(k.hdx[d] * ig2, vn[d], o[d]);
+        o[d] = fmaf(h.hdx[d] * ig2, vn[d], o[d]);
         const float before = vn[d];
-        leaving |= move_mixed(c, b, k, d, o[d], ci[d], rel[d], vn[d]);
+        leaving |= move_mixed(c, b, k.dim[d], n[d], d, o[d], ci[d], rel[d], vn[d]);
         if (vn[d] != before)
             rq[d] = -rq[d];
     }
@@ -732,12 +734,12 @@ __device__ __forceinline__ float push_one(const Ctx &c, const BoxDev &b, const M
     }
 
     if (FULL)
-        deposit_moments_one<D>(c, b, k, ci, rel, o, vn, ig2, sD, mout);
+        deposit_moments_one<D>(c, b, h, k, ci, rel, o, vn, ig2, sD, mout);
 
     if (!isfinite(vn[0] + vn[1] + vn[2]))
         set_status(c.status, MHDPIC_ST_NONFINITE);
-    const int row = D == 3 ? ci[2] * k.n[1] + ci[1] : ci[1];
-    store_particle(c, j, row * k.n[0] + ci[0], o, vn, res_pack(rq));
+    const int row = D == 3 ? ci[2] * n4.y + ci[1] : ci[1];
+    store_particle(c, j, row * n4.x + ci[0], o, vn, res_pack(rq));
     return vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2];
 }
 
@@ -803,7 +805,7 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
         fence_proxy_async();   // the last reads of the tile ended at a barrier before
         mbar_expect_tx(&s_bar, copy_bytes);
         const unsigned char *tm = c.tmaps + (size_t)it.box * 256;
-        const int x0 = k.org[0] + FGHOST, y0 = k.org[1] + FGHOST, z0 = k.org[2] + FGHOST;
+        const int x0 = k.dim[0].x + FGHOST, y0 = k.dim[1].x + FGHOST, z0 = k.dim[2].x + FGHOST;
         tma_tile<D>(sFa, tm, 4 * x0, y0, z0, &s_bar);
         tma_tile<D>(sFb, tm + 128, 2 * x0, y0, z0, &s_bar);
     };
@@ -862,27 +864,27 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
                 int tx, ty, tz;
                 tile_cell(c, t, tx, ty, tz);
                 // the tile lies inside the padded planes (they cover the brick grid plus the halo)
-                const int64_t f = fidx(b, k.org[0] + tx, k.org[1] + ty, k.org[2] + tz);
+                const int64_t f = fidx(b, k.dim[0].x + tx, k.dim[1].x + ty, k.dim[2].x + tz);
                 const int sl = tx + c.fts[1] * ty + c.fts[2] * tz;
                 sFa[sl] = __ldg(c.fa + f);
                 sFb[sl] = __ldg(c.fb + f);
             }
             __syncthreads();
         }
-        // the item constants stay in shared memory where registers are short
+        const HotConst h = s_k[q].h;
         MixedConst kreg;
-        if (!CONST_IN_SMEM<D>)
+        if (!INTS_IN_SMEM<D>)
             kreg = s_k[q];
-        const MixedConst &k = CONST_IN_SMEM<D> ? s_k[q] : kreg;
+        const MixedConst &k = INTS_IN_SMEM<D> ? s_k[q] : kreg;
 
         float vm2 = 0.f;
         {
             const LaneRange lr = lane_range(it, wid, NW);
             const int lane0 = lane * lr.q, re = min(lr.q, lr.cnt - lane0), rs = lr.stride;   // this lane's rounds end at re
-            // source particle of sorted position base + (lane0 + r) step; when the
-            // push applies a sort the permutation entry is loaded one
-            // iteration early.  (One code path for both cases, so that the
-            // arithmetic is the same instruction for instruction.)
+            // source particle of sorted position base + r step (base the lane's
+            // first); when the push applies a sort the permutation entry is
+            // loaded ahead of the records.  (One code path for both cases, so
+            // that the arithmetic is the same instruction for instruction.)
             const bool gather = c.perm_src != nullptr;
             const int base = lr.base + lane0 * lr.step;
             auto src_of = [&](int r) {
@@ -910,18 +912,23 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
                     cp_async_commit();
                     cp_async_wait_prev();
                     if (r < re)
-                        vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, k, base + r * lr.step, load_staged(ring + st * RS),
+                        vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, h, k, base + r * lr.step, load_staged(ring + st * RS),
                                                            sFa, sFb, sD, mout));
                     st = st + 1 == NS ? 0 : st + 1;
                 }
             } else {
-                int sn = lr.first < re ? src_of(lr.first) : 0;
+                // the next particle's records and the place of the one after it
+                PIn nx{};
+                if (lr.first < re)
+                    nx = load_global(c, src_of(lr.first));
+                int sn = lr.first + rs < re ? src_of(lr.first + rs) : 0;
                 for (int r = lr.first; r < re; r += rs) {
-                    const int src = sn;
+                    const PIn pin = nx;
                     if (r + rs < re)
-                        sn = src_of(r + rs);
-                    vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, k, base + r * lr.step, load_global(c, src), sFa, sFb, sD,
-                                                       mout));
+                        nx = load_global(c, sn);
+                    if (r + 2 * rs < re)
+                        sn = src_of(r + 2 * rs);
+                    vm2 = fmaxf(vm2, push_one<D, FULL>(c, b, h, k, base + r * lr.step, pin, sFa, sFb, sD, mout));
                 }
             }
         }
@@ -1093,12 +1100,12 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_deposit_mixed(Ctx c, const Wor
                 if (pin.cell == DEAD_CELL)
                     continue;
                 int ci[3], rel[3] = {0, 0, 0};
-                decode_item_cell<D>(k, pin.cell, ci);
+                decode_item_cell<D>(k.n, k.div, pin.cell, ci);
 #pragma unroll
                 for (int d = 0; d < D; ++d)
-                    rel[d] = tile_coord(k, d, ci[d]);
-                const float ig = rsqrtf(fmaf(vsq3(pin.v), k.invC2, 1.f));
-                deposit_moments_one<D>(c, b, k, ci, rel, pin.o, pin.v, ig, sD, mout);
+                    rel[d] = tile_coord(k.dim[d], ci[d]);
+                const float ig = rsqrtf(fmaf(vsq3(pin.v), k.h.invC2, 1.f));
+                deposit_moments_one<D>(c, b, k.h, k, ci, rel, pin.o, pin.v, ig, sD, mout);
             }
         }
         __syncthreads();

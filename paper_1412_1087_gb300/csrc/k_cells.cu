@@ -247,10 +247,13 @@ int grid_for(int64_t n, int threads)
 
 int launch_prep(const Ctx &c, int cur, int apply, cudaStream_t st)
 {
+    // small boxes: a block for every 32 cells (see prep_cells)
+    const int64_t groups = (c.nc + 31) / 32;
+    const int grid = groups <= 152 * 8 ? (int)(groups < 1 ? 1 : groups) : grid_for(c.nc, 256);
     if (c.prec == MHDPIC_PREC_MIXED)
-        k_prep<MHDPIC_PREC_MIXED><<<grid_for(c.nc, 256), 256, 0, st>>>(c, cur, apply);
+        k_prep<MHDPIC_PREC_MIXED><<<grid, 256, 0, st>>>(c, cur, apply);
     else
-        k_prep<MHDPIC_PREC_FP64><<<grid_for(c.nc, 256), 256, 0, st>>>(c, cur, apply);
+        k_prep<MHDPIC_PREC_FP64><<<grid, 256, 0, st>>>(c, cur, apply);
     return 1;
 }
 

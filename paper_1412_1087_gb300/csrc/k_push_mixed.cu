@@ -107,12 +107,17 @@ struct Wts {
 
 // The constants of an item, by the first 32 threads of the block: a lane per
 // channel, per dimension and for the rest (one thread computing all of them
-// kept the block waiting 2 to 3 us an item).
-__device__ __forceinline__ void item_const(const Ctx &c, const BoxDev &b, const ItemGeom &gm, float dt, int D,
+// kept the block waiting 2 to 3 us an item).  Those of the channels depend on
+// the corrector scales, the others (ITEM_BOX) on the box and the item alone.
+enum { ITEM_SCALES = 1, ITEM_BOX = 2 };
+
+__device__ __forceinline__ void item_const(const BoxDev &b, const ItemGeom &gm, float dt, int D, int which,
                                            MixedConst &k)
 {
     const int l = threadIdx.x;
     if (l < NCH) {
+        if (!(which & ITEM_SCALES))
+            return;
         const float wmax = D == 3 ? 0.421875f : 0.5625f;   // largest TSC weight of one cell
         // sized for the largest item, so that every item of a box has the same
         // tile scale and a contribution rounds the same whichever item holds it
@@ -132,6 +137,8 @@ __device__ __forceinline__ void item_const(const Ctx &c, const BoxDev &b, const 
         k.h.st[l] = ldexpf(1.f, et);
         k.gs[l] = ldexpf(1.f, eg);
         k.h.qb[l] = Q;
+    } else if (!(which & ITEM_BOX)) {
+        return;
     } else if (l < NCH + 3) {
         const int d = l - NCH;
         const int n = b.n[d], centre = gm.half[d] + HALO;
@@ -767,13 +774,17 @@ __device__ __forceinline__ void tma_tile(void *dst, const unsigned char *tmap, i
                      : "memory");
 }
 
-// The push over the work items of the last sort, taken from an atomic
-// counter by the calling kernel's persistent blocks (smem: the dynamic shared
-// memory, push_smem_bytes_mixed bytes).
-template <int D, bool FULL>
-__device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restrict__ items, const int nit,
+// The push over the work items of the last sort: each persistent block of the
+// calling kernel starts with the item of its own number and takes the others
+// from an atomic counter (smem: the dynamic shared memory,
+// push_smem_bytes_mixed bytes).
+// `ready` is called by all threads once the block's first item is being set up
+// and before anything that depends on the corrector scales; where it returns
+// false the push ends and returns false.
+template <int D, bool FULL, typename Ready>
+__device__ __forceinline__ bool push_items(const Ctx &c, const WorkItem *__restrict__ items, const int nit,
                                            int32_t *__restrict__ work_ctr, int cur_out, float dt,
-                                           unsigned char *smem)
+                                           unsigned char *smem, Ready ready)
 {
     const int S = c.tile_slots;
     const PushLayout lay = push_layout(S, c.ftile_slots);
@@ -810,13 +821,13 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
         tma_tile<D>(sFb, tm + 128, 2 * x0, y0, z0, &s_bar);
     };
     // warp 0: the entry and the constants of item number `item` into buffer q
-    auto fetch_item = [&](int item, int q) {
+    auto fetch_item = [&](int item, int q, int which) {
         if (lane == 0)
             s_item[q] = item;
         if (item < nit) {
             const WorkItem it = items[item];
             const BoxDev &b = c.boxes[it.box];
-            item_const(c, b, item_geom(c, b, it.brick, D), dt, D, s_k[q]);
+            item_const(b, item_geom(c, b, it.brick, D), dt, D, which, s_k[q]);
             if (lane == 0)
                 s_it[q] = it;
         }
@@ -829,16 +840,21 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
             z[s] = make_int4(0, 0, 0, 0);
     };
 
+    const int first = blockIdx.x;
     if (wid == 0) {
-        int first = 0;
-        if (lane == 0)
-            first = atomicAdd(work_ctr, 1);
-        fetch_item(__shfl_sync(0xffffffffu, first, 0), 0);
+        fetch_item(first, 0, ITEM_BOX);
         __syncwarp();
-        if (c.tma && lane == 0 && s_item[0] < nit)
+        if (c.tma && lane == 0 && first < nit)
             copy_fields(s_it[0], s_k[0]);
     }
     clear_tile();
+    if (!ready()) {
+        if (c.tma && first < nit)   // the copies in flight have their time
+            mbar_wait(&s_bar, phase, COPY_LIMIT_NS);
+        return false;
+    }
+    if (wid == 0 && first < nit)
+        fetch_item(first, 0, ITEM_SCALES);
     __syncthreads();
 
     for (int q = 0;; q ^= 1) {
@@ -848,14 +864,14 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
         const BoxDev &b = c.boxes[it.box];
         int next = 0;
         if (threadIdx.x == 0)
-            next = atomicAdd(work_ctr, 1);   // used after the particles
+            next = (int)gridDim.x + atomicAdd(work_ctr, 1);   // used after the particles
         if (c.tma) {
             const bool ok = mbar_wait(&s_bar, phase, c.copy_limit_ns);
             if (__syncthreads_or(!ok)) {   // give up the launch, after the copies in flight have had their time
                 if (threadIdx.x == 0)
                     set_status(c.status, MHDPIC_ST_COPY_TIMEOUT);
                 mbar_wait(&s_bar, phase, COPY_LIMIT_NS);
-                return;
+                return true;
             }
             phase ^= 1u;
         } else {
@@ -936,7 +952,7 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
         if (lane == 0 && vb)
             atomicMax(&c.stats[it.box].vmax, vb);
         if (wid == 0)
-            fetch_item(__shfl_sync(0xffffffffu, next, 0), q ^ 1);
+            fetch_item(__shfl_sync(0xffffffffu, next, 0), q ^ 1, ITEM_SCALES | ITEM_BOX);
         __syncthreads();
         // the fields of the next item land while this one is flushed
         if (c.tma && threadIdx.x == 0 && s_item[q ^ 1] < nit)
@@ -967,6 +983,7 @@ __device__ __forceinline__ void push_items(const Ctx &c, const WorkItem *__restr
         clear_tile();
         __syncthreads();
     }
+    return true;
 }
 
 template <int D, bool FULL>
@@ -976,7 +993,10 @@ __global__ void __launch_bounds__(PUSH_THREADS, MIN_BLOCKS<D>) k_push_mixed(Ctx 
                                                                  float dt)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    push_items<D, FULL>(c, items, *nitems, work_ctr, cur_out, dt, smem);
+    push_items<D, FULL>(c, items, *nitems, work_ctr, cur_out, dt, smem, [] {
+        __syncthreads();   // the first item's entry
+        return true;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1019,7 +1039,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *bar, unsigned nblocks, lo
                     ok = 0;
                     break;
                 }
-                __nanosleep(128);
+                __nanosleep(20);
             }
         }
         __threadfence();
@@ -1036,16 +1056,17 @@ __global__ void __launch_bounds__(PUSH_THREADS, MIN_BLOCKS<D>) k_step_mixed(Ctx 
                                                                  double dt, GridBarrier *bar, long long limit_ns)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    if (blockIdx.x == 0) {   // the corrector scales, and the push's work counter
-        for (int bx = threadIdx.x; bx < c.nbox; bx += blockDim.x)
-            scales_box(c, bx, dt);
-        if (threadIdx.x == 0)
-            *work_ctr = 0;
-    }
-    if (!grid_sync(bar, gridDim.x, limit_ns, c.status))
-        return;
-    push_items<D, true>(c, items, *nitems, work_ctr, cur ^ 1, dtf, smem);
-    if (!grid_sync(bar, gridDim.x, limit_ns, c.status))
+    // the blocks set up their first item beside the corrector scales
+    const bool pushed = push_items<D, true>(c, items, *nitems, work_ctr, cur ^ 1, dtf, smem, [&] {
+        if (blockIdx.x == 0) {   // the corrector scales, and the push's work counter
+            for (int bx = threadIdx.x; bx < c.nbox; bx += blockDim.x)
+                scales_box(c, bx, dt);
+            if (threadIdx.x == 0)
+                *work_ctr = 0;
+        }
+        return grid_sync(bar, gridDim.x, limit_ns, c.status);
+    });
+    if (!pushed || !grid_sync(bar, gridDim.x, limit_ns, c.status))
         return;
     prep_cells<MHDPIC_PREC_MIXED>(c, cur ^ 1, 1);
 }
@@ -1086,7 +1107,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_deposit_mixed(Ctx c, const Wor
         for (int s = threadIdx.x; s < TILE_WORDS * S; s += PUSH_THREADS)
             sD[s] = 0;
         if (threadIdx.x < 32)
-            item_const(c, b, gm, 0.f, D, s_k);
+            item_const(b, gm, 0.f, D, ITEM_SCALES | ITEM_BOX, s_k);
         __syncthreads();
         const MixedConst &k = s_k;
         {

@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
     __shared__ int s_item;
     __shared__ F64Const s_k;
     unsigned long long *mout = c.momdep[cur_out];
-    const int nit = *nitems;
+    const int nfront = nitems[0], nit = nfront + nitems[1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int NW = PUSH_THREADS / 32;
 
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
         const int item = s_item;
         if (item >= nit)
             break;
-        const WorkItem it = items[item];
+        const WorkItem it = work_item(c, items, nfront, item);
         const BoxDev &b = c.boxes[it.box];
         const ItemGeom gm = item_geom(c, b, it.brick, D);
 

@@ -782,10 +782,11 @@ __device__ __forceinline__ void tma_tile(void *dst, const unsigned char *tmap, i
 // and before anything that depends on the corrector scales; where it returns
 // false the push ends and returns false.
 template <int D, bool FULL, typename Ready>
-__device__ __forceinline__ bool push_items(const Ctx &c, const WorkItem *__restrict__ items, const int nit,
-                                           int32_t *__restrict__ work_ctr, int cur_out, float dt,
-                                           unsigned char *smem, Ready ready)
+__device__ __forceinline__ bool push_items(const Ctx &c, const WorkItem *__restrict__ items,
+                                           const int32_t *__restrict__ nitems, int32_t *__restrict__ work_ctr,
+                                           int cur_out, float dt, unsigned char *smem, Ready ready)
 {
+    const int nfront = nitems[0], nit = nfront + nitems[1];
     const int S = c.tile_slots;
     const PushLayout lay = push_layout(S, c.ftile_slots);
     int *sD = reinterpret_cast<int *>(smem);
@@ -825,7 +826,7 @@ __device__ __forceinline__ bool push_items(const Ctx &c, const WorkItem *__restr
         if (lane == 0)
             s_item[q] = item;
         if (item < nit) {
-            const WorkItem it = items[item];
+            const WorkItem it = work_item(c, items, nfront, item);
             const BoxDev &b = c.boxes[it.box];
             item_const(b, item_geom(c, b, it.brick, D), dt, D, which, s_k[q]);
             if (lane == 0)
@@ -993,7 +994,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, MIN_BLOCKS<D>) k_push_mixed(Ctx 
                                                                  float dt)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    push_items<D, FULL>(c, items, *nitems, work_ctr, cur_out, dt, smem, [] {
+    push_items<D, FULL>(c, items, nitems, work_ctr, cur_out, dt, smem, [] {
         __syncthreads();   // the first item's entry
         return true;
     });
@@ -1057,7 +1058,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, MIN_BLOCKS<D>) k_step_mixed(Ctx 
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // the blocks set up their first item beside the corrector scales
-    const bool pushed = push_items<D, true>(c, items, *nitems, work_ctr, cur ^ 1, dtf, smem, [&] {
+    const bool pushed = push_items<D, true>(c, items, nitems, work_ctr, cur ^ 1, dtf, smem, [&] {
         if (blockIdx.x == 0) {   // the corrector scales, and the push's work counter
             for (int bx = threadIdx.x; bx < c.nbox; bx += blockDim.x)
                 scales_box(c, bx, dt);
@@ -1089,7 +1090,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_deposit_mixed(Ctx c, const Wor
     __shared__ int s_item;
     __shared__ MixedConst s_k;
     unsigned long long *mout = c.momdep[cur];
-    const int nit = *nitems;
+    const int nfront = nitems[0], nit = nfront + nitems[1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int NW = PUSH_THREADS / 32;
     const bool gather = c.perm_src != nullptr;
@@ -1101,7 +1102,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_deposit_mixed(Ctx c, const Wor
         const int item = s_item;
         if (item >= nit)
             break;
-        const WorkItem it = items[item];
+        const WorkItem it = work_item(c, items, nfront, item);
         const BoxDev &b = c.boxes[it.box];
         const ItemGeom gm = item_geom(c, b, it.brick, D);
         for (int s = threadIdx.x; s < TILE_WORDS * S; s += PUSH_THREADS)

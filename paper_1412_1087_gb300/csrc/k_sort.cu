@@ -508,7 +508,10 @@ __device__ __forceinline__ int brick_items(const Ctx &c, int cnt, int na)
 
 // The push work list, SORT_THREADS consecutive bricks per block and pass:
 // their items go to a range of the list that the block reserves (the order of
-// the ranges does not matter: the deposits are integer sums).
+// the ranges does not matter: the deposits are integer sums).  Bricks of less
+// than item_big particles (the ragged edge of a box, sparse regions) go to the
+// far end of the array, backwards, and are pushed last (work_item), where they
+// fill the blocks that run out first.
 constexpr int SORT_THREADS = 256;
 
 __device__ __forceinline__ void write_items(const Ctx &c, const int64_t *__restrict__ brick_start,
@@ -516,7 +519,7 @@ __device__ __forceinline__ void write_items(const Ctx &c, const int64_t *__restr
                                             int32_t *__restrict__ nitems, int block, int nblocks)
 {
     __shared__ int ws[32];
-    __shared__ int s_first;
+    __shared__ int s_first[2];
     const int vol = c.brick[0] * c.brick[1] * c.brick[2];
     for (int64_t g0 = (int64_t)block * SORT_THREADS; g0 < c.nbricks_total; g0 += (int64_t)nblocks * SORT_THREADS) {
         const int64_t gb = g0 + threadIdx.x;
@@ -533,12 +536,16 @@ __device__ __forceinline__ void write_items(const Ctx &c, const int64_t *__restr
             pm = c.halves ? (int64_t)offset[k0 + vol / 2] : w.p1;
             m = brick_items(c, (int)(w.p1 - w.p0), (int)(pm - w.p0));
         }
-        int tot;
-        const int pre = block_exclusive_scan(m, ws, &tot);
-        if (threadIdx.x == 0)
-            s_first = tot > 0 ? atomicAdd(nitems, tot) : 0;
+        const bool small = m > 0 && w.p1 - w.p0 < c.item_big;
+        int tot, small_tot;
+        const int pre = block_exclusive_scan(small ? 0 : m, ws, &tot);
+        const int small_pre = block_exclusive_scan(small ? m : 0, ws, &small_tot);
+        if (threadIdx.x == 0) {
+            s_first[0] = tot > 0 ? atomicAdd(nitems, tot) : 0;
+            s_first[1] = small_tot > 0 ? atomicAdd(nitems + 1, small_tot) : 0;
+        }
         __syncthreads();
-        int o = s_first + pre;
+        int64_t o = small ? c.items_size - 1 - (s_first[1] + small_pre) : s_first[0] + pre;
         if (m > 0 && w.p1 - w.p0 <= c.item_cap) {
             // one item; a whole 64-cell brick splits at its 32nd cell (the
             // start of the second half)

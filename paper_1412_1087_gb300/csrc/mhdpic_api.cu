@@ -743,13 +743,20 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     c->grid_blocks = bps * (nsm > 0 ? nsm : 1);
-    // work items: a brick's particles, but no more than there are for each
-    // resident block where that is less than a brick (small boxes leave SMs
-    // idle otherwise: 64 bricks of 1,024 particles at 64^2 x 16), in whole
-    // rounds of the block's threads
-    k.item_cap = (int32_t)std::min<int64_t>(
-        ITEM_MAX_PARTICLES,
-        std::max<int64_t>(1, (np / c->grid_blocks + PUSH_THREADS - 1) / PUSH_THREADS) * PUSH_THREADS);
+    // work items: a brick's particles, but where there are fewer bricks than
+    // resident blocks (small boxes leave SMs idle otherwise: 64 bricks of
+    // 1,024 particles at 64^2 x 16) no more than there are for each block, in
+    // whole rounds of the block's threads.  (Bricks cut up where there are
+    // more than blocks only make more items to set up: 336 bricks of 512
+    // particles in 3-D 54 us a push whole, 70 with half of them cut in two.)
+    k.item_cap = ITEM_MAX_PARTICLES;
+    if (k.nbricks_total < c->grid_blocks)
+        k.item_cap = (int32_t)std::min<int64_t>(
+            ITEM_MAX_PARTICLES,
+            std::max<int64_t>(1, (np / c->grid_blocks + PUSH_THREADS - 1) / PUSH_THREADS) * PUSH_THREADS);
+    // items below three quarters of the mean brick go last
+    k.item_big = (int32_t)std::min<int64_t>(k.item_cap / 2, 3 * np / (4 * k.nbricks_total));
+    k.items_size = 2 * k.nbricks_total + np / k.item_cap + 2;
 
     // device allocations
     BoxDev *boxes_d;
@@ -788,7 +795,7 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
         (rc = c->alloc((char **)&c->s.tmp, (size_t)np * c->particle_bytes())) ||
         // at most one item per brick, or per half of a crowded brick
         // ceil(n_half / item_cap) <= n_half / item_cap + 1
-        (rc = c->alloc(&c->s.items, 2 * k.nbricks_total + np / k.item_cap + 2)) ||
+        (rc = c->alloc(&c->s.items, (size_t)k.items_size)) ||
         (rc = c->alloc(&c->s.max_count, 1)) ||
         (rc = c->alloc(&c->work_ctr, 1)))
         return bail(rc);

@@ -130,6 +130,8 @@ struct Ctx {
     int32_t ftile_slots;   // slots of the field tile
     int32_t tma;           // 1: field tiles staged by tensor copies (tmaps), 0: by the threads
     int32_t item_cap;      // particles of a work item, at most
+    int32_t item_big;      // bricks of at least so many come first in the work list (at most item_cap)
+    int64_t items_size;    // entries of the work list
     int32_t halves;        // 1: default 64-cell bricks split into 32-cell halves
     double sort_ahead;     // sort key: the cell after moving for this time at the current velocity
     const float4 *sort_k;  // per box {t/dx, t/dy, t/dz, 1/C^2} in FP32 for that key
@@ -178,7 +180,7 @@ struct Ctx {
 // launchers (each returns the number of kernel launches it made, or -1 on a
 // launch error; the caller checks cudaGetLastError)
 // ---------------------------------------------------------------------------
-constexpr int SORT_COUNTERS = 3;   // counters kept after the counts, cleared with them
+constexpr int SORT_COUNTERS = 4;   // counters kept after the counts, cleared with them
 struct SortScratch {
     int32_t *count;     // [nkeys + 2], then long_count and nitems
     int32_t *offset;    // [nkeys + 1]
@@ -191,7 +193,7 @@ struct SortScratch {
     void *tmp;          // particle staging, np * (largest particle record)
     int64_t *brick_start;  // device [nbox + 1] first global brick of each box
     WorkItem *items;
-    int32_t *nitems;       // [1]
+    int32_t *nitems;       // [2] items from the list's front, and from its end
     int32_t *max_count;    // [1]
 };
 

@@ -19,6 +19,13 @@ __device__ __forceinline__ bool removed_early(const Ctx &c, int64_t j)
     return ti < c.clock[1] && c.clock[0] >= 2.0 * ti;
 }
 
+// Entry i of the work list: the first nitems[0] from its front, the rest
+// backwards from its end.
+__device__ __forceinline__ WorkItem work_item(const Ctx &c, const WorkItem *__restrict__ items, int nfront, int i)
+{
+    return items[i < nfront ? i : c.items_size - 1 - (i - nfront)];
+}
+
 struct ItemGeom {
     int org[3];    // unwrapped box coordinates of tile cell (0,0,0)
     int ctr[3];    // brick centre, for periodic unwrapping of particle cells

@@ -14,7 +14,7 @@
 // integer products (wide_fixed.cuh), gamma and 1/gamma come from one
 // reciprocal square root (math64.cuh) instead of square roots and divisions,
 // positions are compared and cut into cell and offset with integer
-// operations: at 48^3 x 16 particles 4.40 -> 2.43 ms a push (1100 -> 440 FP64
+// operations: at 48^3 x 16 particles 4.40 -> 2.25 ms a push (1100 -> 440 FP64
 // operations a particle; the FP64 pipe is now 54% busy, and the shared 64-bit
 // atomics, compare-and-swap loops, are the longest waits).
 #include "math64.cuh"
@@ -81,9 +81,11 @@ __device__ __forceinline__ void gather_f64(const Ctx &c, const BoxDev &b, bool i
     int gx[3], gy[3], gz[3];
     if (!in_tile)
         stencil_coords<D>(b, ci, gx, gy, gz);
+    // rolled: the code of a whole particle, unrolled, misses the instruction
+    // cache (7% of the push, with the deposit a function of its own)
 #pragma unroll 1
     for (int cz = 0; cz < (D == 3 ? 3 : 1); ++cz)
-#pragma unroll
+#pragma unroll 1
         for (int cy = 0; cy < 3; ++cy) {
             const double wyz = D == 3 ? w[1][cy] * w[2][cz] : w[1][cy];
 #pragma unroll
@@ -116,7 +118,7 @@ __device__ __forceinline__ void cell_of_f64(const F64Const &k, const double x[3]
 // into the tile when the stencil lies in it, else into the global
 // accumulators; the same integers either way.
 template <int D>
-__device__ __forceinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in_tile, int base, const int ci[3],
+__device__ __noinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in_tile, int base, const int ci[3],
                                              const double o[3], const double q[4],
                                              unsigned long long *__restrict__ sD,
                                              unsigned long long *__restrict__ gdst)

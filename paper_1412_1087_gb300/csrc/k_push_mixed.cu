@@ -9,10 +9,10 @@
 //  * Lanes and cells: a 64-cell brick is two 32-cell halves; warps 0-3 work
 //    on one half and warps 4-7 on the other, and lane l takes the l-th 1/32 of
 //    its half's (cell-sorted) particles, so the 32 lanes of an instruction sit
-//    in about 32 different cells.  The tile strides are padded (3-D: y 12,
-//    z 112 slots; 2-D: y 24) so that 32 cells of a half fall on 32 different
-//    banks for the 32-bit deposit atomics and on distinct bank groups for the
-//    128-bit and 64-bit field loads.  (Giving each lane exactly one cell's
+//    in about 32 different cells.  The tile strides are padded (3-D: y 8,
+//    z 68 slots; 2-D: y 24) so that 32 cells of a half fall on 32 different
+//    banks for the 32-bit deposit atomics, the field tile's (y 12, z dense) on
+//    distinct bank groups for the 128-bit and 64-bit field loads.  (Giving each lane exactly one cell's
 //    particles removes more conflicts but idles a quarter of the lanes, since
 //    cell counts vary; the even split measured 11% faster.)
 //  * Fixed point in the tile: each contribution x = a w (in tile units, the
@@ -1166,14 +1166,31 @@ int occupancy_all(size_t bytes)
     return occupancy_mixed<D, true>(bytes);
 }
 
+// The push takes no more shared memory from the SM's 228 KB than its resident
+// blocks need: the 3-D particle records come through L1, and an SM that the
+// kernel before left with more shared memory would stay so (two steps of
+// 128^3 x 32 with three contexts at work 21.7 ms without, 21.2 with; alone the
+// same 21.4).
 template <int D>
 void launch_d(const Ctx &c, const SortScratch &s, int32_t *work_ctr, int cur_out, int full, float dt, int grid,
               size_t bytes, cudaStream_t st)
 {
-    if (full)
-        k_push_mixed<D, true><<<grid, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
-    else
-        k_push_mixed<D, false><<<grid, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
+    const size_t need = (size_t)MIN_BLOCKS<D> * (bytes + sizeof(MixedConst) * 2 + 1280);
+    const size_t percent = (need * 100 + 228 * 1024 - 1) / (228 * 1024);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(PUSH_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[0].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const WorkItem *items = s.items;
+    const int32_t *nitems = s.nitems;
+    cudaLaunchKernelEx(&cfg, full ? k_push_mixed<D, true> : k_push_mixed<D, false>, c, items, nitems, work_ctr, cur_out,
+                       dt);
 }
 
 }  // namespace

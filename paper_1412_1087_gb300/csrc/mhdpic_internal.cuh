@@ -126,7 +126,7 @@ struct Ctx {
     FastDiv tdx, tdxy;     // division by tile[0] and tile[0] tile[1]
     int32_t ts[3];         // tile strides in slots (x, y, z); padded to spread banks
     int32_t tile_slots;    // slots of the tile (>= tile_vol)
-    int32_t fts[3];        // field tile strides (x 1, y ts[1], z dense): the layout a tensor copy writes
+    int32_t fts[3];        // field tile strides (z dense): the layout a tensor copy writes
     int32_t ftile_slots;   // slots of the field tile
     int32_t tma;           // 1: field tiles staged by tensor copies (tmaps), 0: by the threads
     int32_t item_cap;      // particles of a work item, at most

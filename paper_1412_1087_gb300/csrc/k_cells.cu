@@ -190,9 +190,9 @@ __global__ void k_velocities_to_double(Ctx c, double *__restrict__ out)
     }
 }
 
-// Largest |v| per box (for the fixed-point scales): a running maximum per
+// FP64 precision: largest |v| per box (for the fixed-point scales; in mixed
+// precision the deposit records it): a running maximum per
 // thread while its particles stay in one box, one atomic per box and warp.
-template <int PREC>
 __global__ void k_vmax(Ctx c)
 {
     float acc = 0.f;
@@ -207,19 +207,12 @@ __global__ void k_vmax(Ctx c)
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c.np;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int bx = find_box(c.box_part_start, c.nbox, i);
-        float vm;
-        if (PREC == MHDPIC_PREC_MIXED) {
-            const float4 vs = c.vel[i];
-            const float v[3] = {vs.x, vs.y, vs.z};
-            vm = sqrtf(vsq3(v));
-        } else {
-            double v2 = 0.0;
-            for (int d = 0; d < 3; ++d) {
-                const double v = c.p64[(int64_t)d * c.np + i];
-                v2 += v * v;
-            }
-            vm = (float)sqrt(v2);
+        double v2 = 0.0;
+        for (int d = 0; d < 3; ++d) {
+            const double v = c.p64[(int64_t)d * c.np + i];
+            v2 += v * v;
         }
+        float vm = (float)sqrt(v2);
         if (!(vm <= 1.0e37f))
             vm = 1.0e37f;
         if (bx != bacc) {   // rare: a thread's particles cross into the next box
@@ -306,10 +299,7 @@ int launch_vmax(const Ctx &c, cudaStream_t st)
 {
     if (c.np == 0)
         return 0;
-    if (c.prec == MHDPIC_PREC_MIXED)
-        k_vmax<MHDPIC_PREC_MIXED><<<grid_for(c.np, 256), 256, 0, st>>>(c);
-    else
-        k_vmax<MHDPIC_PREC_FP64><<<grid_for(c.np, 256), 256, 0, st>>>(c);
+    k_vmax<<<grid_for(c.np, 256), 256, 0, st>>>(c);
     return 1;
 }
 

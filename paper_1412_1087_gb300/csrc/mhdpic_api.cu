@@ -510,7 +510,8 @@ int do_sort(mhdpic_ctx *c, int64_t *perm_out, int32_t *counts_out)
     return copy_particles(c, false);
 }
 
-// Charge/current deposit of the current particles into moments buffer cur.
+// Charge/current deposit of the current particles into moments buffer cur, and
+// their largest |v| per box.
 // Mixed precision goes through the push's tile over the work list of a sort
 // of the current particles: the list is current when `listed` (right after
 // a sort that has been applied), else a pending sort is used or one is made
@@ -519,9 +520,9 @@ int deposit_current(mhdpic_ctx *c, bool listed)
 {
     int rc;
     if (c->k.prec != MHDPIC_PREC_MIXED) {
-        if ((rc = materialize(c)))
+        if ((rc = materialize(c)) || (rc = check_launch(c, launch_moments(c->k, c->cur, c->stream))))
             return rc;
-        return check_launch(c, launch_moments(c->k, c->cur, c->stream));
+        return check_launch(c, launch_vmax(c->k, c->stream));
     }
     Ctx kk = c->k;
     if (!listed) {
@@ -926,8 +927,7 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
 
     // moments at the initial positions, maxima, staged fields
     c->cur = 0;
-    if ((rc = deposit_current(c, true)) || (rc = check_launch(c, launch_vmax(k, st))) ||
-        (rc = do_prep(c, 0)))
+    if ((rc = deposit_current(c, true)) || (rc = do_prep(c, 0)))
         return bail(rc);
     if ((rc = copy_particles(c, false)))
         return bail(rc);
@@ -1030,8 +1030,7 @@ int mhdpic_deposit(mhdpic_ctx *c)
     if ((rc = copy_particles(c, true)) || (rc = copy_gas(c, true, true)))
         return rc;
     // the stage kernel clears buffer cur^1, so deposit into cur and stage from it
-    if ((rc = deposit_current(c, false)) || (rc = check_launch(c, launch_vmax(c->k, c->stream))) ||
-        (rc = do_prep(c, 0)))
+    if ((rc = deposit_current(c, false)) || (rc = do_prep(c, 0)))
         return rc;
     return MHDPIC_OK;
 }

@@ -220,6 +220,7 @@ int launch_max_count(const Ctx &c, const SortScratch &s, cudaStream_t st);
 int launch_mark_free(const Ctx &c, const SortScratch &s, cudaStream_t st);
 // number of particles that have not left the box (into out, device)
 int launch_count_live(const Ctx &c, unsigned long long *out, cudaStream_t st);
+// FP64 precision: the largest |v| per box
 int launch_vmax(const Ctx &c, cudaStream_t st);
 int launch_prep(const Ctx &c, int cur, int apply, cudaStream_t st);
 // FP64 precision: charge and current at the current positions into momdep[cur]
@@ -230,7 +231,7 @@ int launch_push_f64(const Ctx &c, const SortScratch &s, int32_t *work_ctr, int c
                     double dt, int grid_blocks, cudaStream_t st);
 // mixed precision: charge/current deposit at the stored positions through the
 // push's tile, over the work list of the last sort (particles read through
-// c.perm_src when set); momdep[cur] must be zero
+// c.perm_src when set); momdep[cur] must be zero; records the largest |v| per box
 int launch_deposit_mixed(const Ctx &c, const SortScratch &s, int32_t *work_ctr, int cur, int grid_blocks,
                          cudaStream_t st);
 int launch_scales(const Ctx &c, double dt, cudaStream_t st);

@@ -6,7 +6,7 @@
 //
 // Same work decomposition as the mixed kernel (k_push_mixed.cu): persistent
 // CTAs take brick items from an atomic counter, stage the brick's fields plus
-// a halo in shared memory and accumulate the deposits in a shared int64
+// a halo in shared memory and accumulate the deposits in a shared
 // fixed-point tile that is added to the global accumulators at the end; a
 // particle whose stencil leaves the tile uses global memory directly.
 //
@@ -14,9 +14,8 @@
 // integer products (wide_fixed.cuh), gamma and 1/gamma come from one
 // reciprocal square root (math64.cuh) instead of square roots and divisions,
 // positions are compared and cut into cell and offset with integer
-// operations: at 48^3 x 16 particles 4.40 -> 2.25 ms a push (1100 -> 440 FP64
-// operations a particle; the FP64 pipe is now 54% busy, and the shared 64-bit
-// atomics, compare-and-swap loops, are the longest waits).
+// operations (1100 -> 440 FP64 operations a particle); with the deposit tile in
+// 32-bit words a step of 48^3 x 16 particles takes 2.02 ms (4.81 before).
 #include "math64.cuh"
 #include "push_common.cuh"
 #include "wide_fixed.cuh"
@@ -29,6 +28,24 @@ namespace {
 // headroom of the scales), and up to 4 times that before the overflow flag,
 // so q 2^WIDE stays inside int64.
 constexpr int WIDE = 8;
+
+// The deposit tile.  W = 3: a slot is SLOT_WORDS consecutive 32-bit words, three
+// for each channel: 19, 19 and the upper bits of every contribution (an item
+// has at most 4,096 contributions per cell and channel, and they are below
+// 2^55 or, when flagged, go to the global accumulators, so no word overflows
+// before the flush puts them together); an odd slot size keeps slots that differ mod 32 on different banks.  64-bit
+// shared atomic adds are compare-and-swap loops (a step of 48^3 x 16 particles
+// 2.52 ms, 2.02 with three words); they remain (W = 1, a 64-bit word per
+// channel) for bricks whose tile would not fit otherwise.
+constexpr int SLOT_WORDS = 3 * NCH + 1;
+constexpr int WORD_BITS = 19;
+constexpr unsigned WORD_MASK = (1u << WORD_BITS) - 1u;
+
+__host__ __device__ constexpr size_t f64_tile_bytes(int slots, int words)
+{
+    return ((words == 3 ? sizeof(unsigned) * SLOT_WORDS : sizeof(unsigned long long) * NCH) * (size_t)slots + 15) / 16 *
+           16;
+}
 
 struct F64Const {
     double dt, h, C, C2, invC;
@@ -77,7 +94,7 @@ __device__ __forceinline__ void gather_f64(const Ctx &c, const BoxDev &b, bool i
 {
     E[0] = E[1] = E[2] = Bf[0] = Bf[1] = Bf[2] = 0.0;
     const double2 *__restrict__ gF = reinterpret_cast<const double2 *>(c.f64);
-    const int SY = c.ts[1], SZ = c.ts[2];
+    const int SY = c.fts[1], SZ = c.fts[2];
     int gx[3], gy[3], gz[3];
     if (!in_tile)
         stencil_coords<D>(b, ci, gx, gy, gz);
@@ -117,11 +134,10 @@ __device__ __forceinline__ void cell_of_f64(const F64Const &k, const double x[3]
 // Four channels (already at their scales) with the TSC weights of offsets o:
 // into the tile when the stencil lies in it, else into the global
 // accumulators; the same integers either way.
-template <int D>
+template <int D, int W>
 __device__ __noinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in_tile, int base, const int ci[3],
-                                             const double o[3], const double q[4],
-                                             unsigned long long *__restrict__ sD,
-                                             unsigned long long *__restrict__ gdst)
+                                          const double o[3], const double q[4], int ch0, void *sD,
+                                          unsigned long long *__restrict__ gdst)
 {
     const int S = c.tile_slots, SY = c.ts[1], SZ = c.ts[2];
     const int64_t nc = c.nc;
@@ -154,10 +170,19 @@ __device__ __noinline__ void deposit4_f64(const Ctx &c, const BoxDev &b, bool in
         if (in_tile) {
 #pragma unroll
             for (int n = 0; n < 9; ++n) {
-                unsigned long long *t = sD + base + n % 3 + SY * (n / 3) + SZ * cz;
+                const int slot = base + n % 3 + SY * (n / 3) + SZ * cz;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    atomicAdd(t + k * S, wide_value(qz[k], pair[n], sign[k]));
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned long long v = wide_value(qz[k], pair[n], sign[k]);
+                    if (W == 3) {
+                        unsigned *t = static_cast<unsigned *>(sD) + slot * SLOT_WORDS + 3 * (ch0 + k);
+                        atomicAdd(t, (unsigned)v & WORD_MASK);
+                        atomicAdd(t + 1, (unsigned)(v >> WORD_BITS) & WORD_MASK);
+                        atomicAdd(t + 2, (unsigned)((long long)v >> (2 * WORD_BITS)));
+                    } else {
+                        atomicAdd(static_cast<unsigned long long *>(sD) + (ch0 + k) * S + slot, v);
+                    }
+                }
             }
         } else {
 #pragma unroll 1
@@ -189,10 +214,10 @@ __device__ __forceinline__ bool bounded(const BoxDev &b, const F64Const &k, int 
     return boundary_f64(b, d, x, vd);
 }
 
-template <int D, bool FULL>
+template <int D, bool FULL, int W>
 __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, const ItemGeom &gm,
                                               const F64Const &k, int64_t j, const double2 *sF,
-                                              unsigned long long *sD, unsigned long long *mout)
+                                              void *sD, unsigned long long *mout)
 {
     const int64_t np = c.np;
     const int64_t src = c.perm_src ? (int64_t)c.perm_src[j] : j;
@@ -235,6 +260,7 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
     for (int d = 0; d < D; ++d)
         in_tile &= tile_rel(c, b, gm, d, ci[d], rel[d]);
     const int base = (rel[0] - 1) + c.ts[1] * (rel[1] - 1) + (D == 3 ? c.ts[2] * (rel[2] - 1) : 0);
+    const int fbase = (rel[0] - 1) + c.fts[1] * (rel[1] - 1) + (D == 3 ? c.fts[2] * (rel[2] - 1) : 0);
 
     double E[3], Bf[3];
     {
@@ -242,7 +268,7 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
 #pragma unroll
         for (int d = 0; d < D; ++d)
             tsc_from_offset<double>(o[d], w[d]);
-        gather_f64<D>(c, b, in_tile, base, ci, w, sF, E, Bf);
+        gather_f64<D>(c, b, in_tile, fbase, ci, w, sF, E, Bf);
     }
     const double B2 = Bf[0] * Bf[0] + Bf[1] * Bf[1] + Bf[2] * Bf[2];
     if (B2 > 0.0) {
@@ -287,10 +313,11 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
     {
         const double qc[4] = {k.mq[0] * (vn[0] - v[0]), k.mq[1] * (vn[1] - v[1]), k.mq[2] * (vn[2] - v[2]),
                               k.mq[3] * dEk};
-        if (beyond(qc[0], k.vlim[0]) || beyond(qc[1], k.vlim[1]) || beyond(qc[2], k.vlim[2]) ||
-            beyond(qc[3], k.vlim[3]))
+        const bool over = beyond(qc[0], k.vlim[0]) || beyond(qc[1], k.vlim[1]) || beyond(qc[2], k.vlim[2]) ||
+                          beyond(qc[3], k.vlim[3]);
+        if (over)
             set_status(c.status, MHDPIC_ST_OVERFLOW);
-        deposit4_f64<D>(c, b, in_tile, base, ci, o, qc, sD, c.corr);
+        deposit4_f64<D, W>(c, b, in_tile && !over, base, ci, o, qc, CH_MX, sD, c.corr);
     }
 
     {
@@ -319,7 +346,7 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
             in2 &= tile_rel(c, b, gm, d, ci[d], rel2[d]);
         const int base2 = (rel2[0] - 1) + c.ts[1] * (rel2[1] - 1) + (D == 3 ? c.ts[2] * (rel2[2] - 1) : 0);
         const double qm[4] = {k.qn, k.qj[0] * (vn[0] * ig1), k.qj[1] * (vn[1] * ig1), k.qj[2] * (vn[2] * ig1)};
-        deposit4_f64<D>(c, b, in2, base2, ci, o, qm, sD + CH_N * c.tile_slots, mout);
+        deposit4_f64<D, W>(c, b, in2, base2, ci, o, qm, CH_N, sD, mout);
     }
     if (!isfinite(vn[0] + vn[1] + vn[2]))
         set_status(c.status, MHDPIC_ST_NONFINITE);
@@ -334,7 +361,7 @@ __device__ __forceinline__ float push_one_f64(const Ctx &c, const BoxDev &b, con
     return f0 * f0 + f1 * f1 + f2 * f2;
 }
 
-template <int D, bool FULL>
+template <int D, bool FULL, int W>
 __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkItem *__restrict__ items,
                                                           const int32_t *__restrict__ nitems,
                                                           int32_t *__restrict__ work_ctr, int cur_out,
@@ -342,8 +369,11 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int S = c.tile_slots;
-    unsigned long long *sD = reinterpret_cast<unsigned long long *>(smem);
-    double2 *sF = reinterpret_cast<double2 *>(smem + sizeof(unsigned long long) * NCH * S);
+    int4 *clear = reinterpret_cast<int4 *>(smem);
+    const unsigned *sW = reinterpret_cast<const unsigned *>(smem);
+    const unsigned long long *sL = reinterpret_cast<const unsigned long long *>(smem);
+    const size_t tile_bytes = f64_tile_bytes(S, W);
+    double2 *sF = reinterpret_cast<double2 *>(smem + tile_bytes);
     __shared__ int s_item;
     __shared__ F64Const s_k;
     unsigned long long *mout = c.momdep[cur_out];
@@ -362,14 +392,14 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
         const BoxDev &b = c.boxes[it.box];
         const ItemGeom gm = item_geom(c, b, it.brick, D);
 
-        for (int s = threadIdx.x; s < NCH * S; s += PUSH_THREADS)
-            sD[s] = 0ull;
+        for (int s = threadIdx.x; s < (int)(tile_bytes / sizeof(int4)); s += PUSH_THREADS)
+            clear[s] = make_int4(0, 0, 0, 0);
         const double2 *gF = reinterpret_cast<const double2 *>(c.f64);
         for (int t = threadIdx.x; t < c.tile_vol; t += PUSH_THREADS) {
             int tx, ty, tz;
             tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
-            int s = tile_slot(c, tx, ty, tz);
+            const int s = tx + c.fts[1] * ty + c.fts[2] * tz;
             sF[3 * s] = __ldg(gF + 3 * g);
             sF[3 * s + 1] = __ldg(gF + 3 * g + 1);
             sF[3 * s + 2] = __ldg(gF + 3 * g + 2);
@@ -384,7 +414,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
         for (int r = lr.first; r < lr.q; r += lr.stride) {
             const int loc = lane * lr.q + r;
             if (loc < lr.cnt)
-                vm2 = fmaxf(vm2, push_one_f64<D, FULL>(c, b, gm, k, lr.base + loc * lr.step, sF, sD, mout));
+                vm2 = fmaxf(vm2, push_one_f64<D, FULL, W>(c, b, gm, k, lr.base + loc * lr.step, sF, smem, mout));
         }
         unsigned vb = __reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(vm2)));
         if (lane == 0 && vb)
@@ -395,18 +425,19 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
             int tx, ty, tz;
             tile_cell(c, t, tx, ty, tz);
             int64_t g = tile_global(c, b, gm, tx, ty, tz, D);
-            int s = tile_slot(c, tx, ty, tz);
-            for (int ch = 0; ch < 4; ++ch) {
-                unsigned long long a = sD[ch * S + s];
-                if (a)
-                    atomicAdd(c.corr + ch * c.nc + g, a);
-            }
-            if (FULL)
-                for (int ch = 0; ch < 4; ++ch) {
-                    unsigned long long a = sD[(CH_N + ch) * S + s];
-                    if (a)
-                        atomicAdd(mout + ch * c.nc + g, a);
+            const int s = tile_slot(c, tx, ty, tz);
+            for (int ch = 0; ch < (FULL ? NCH : 4); ++ch) {
+                unsigned long long a;
+                if (W == 3) {
+                    const unsigned *t = sW + s * SLOT_WORDS + 3 * ch;
+                    a = (unsigned long long)(long long)(int)t[2] << (2 * WORD_BITS);
+                    a += ((unsigned long long)t[1] << WORD_BITS) + t[0];
+                } else {
+                    a = sL[ch * S + s];
                 }
+                if (a)
+                    atomicAdd(ch < CH_N ? c.corr + ch * c.nc + g : mout + (ch - CH_N) * c.nc + g, a);
+            }
         }
         __syncthreads();
     }
@@ -414,49 +445,47 @@ __global__ void __launch_bounds__(PUSH_THREADS, 2) k_push_f64(Ctx c, const WorkI
 
 constexpr int PUSH_SMEM_LIMIT = 200 * 1024;
 
-template <int D, bool FULL>
-int occupancy_f64(size_t bytes)
+int words_f64(const Ctx &c)
 {
-    cudaFuncSetAttribute(k_push_f64<D, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, PUSH_SMEM_LIMIT);
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_push_f64<D, FULL>, PUSH_THREADS, bytes);
-    return nb;
+    return f64_tile_bytes(c.tile_slots, 3) + 48 * (size_t)c.ftile_slots <= PUSH_SMEM_LIMIT ? 3 : 1;
+}
+
+// the kernel for a context's dimension and tile, with both deposits or the
+// corrector's alone
+auto kernel_f64(const Ctx &c, bool full)
+{
+    const bool w3 = words_f64(c) == 3;
+    if (c.ndim == 3)
+        return full ? (w3 ? k_push_f64<3, true, 3> : k_push_f64<3, true, 1>)
+                    : (w3 ? k_push_f64<3, false, 3> : k_push_f64<3, false, 1>);
+    return full ? (w3 ? k_push_f64<2, true, 3> : k_push_f64<2, true, 1>)
+                : (w3 ? k_push_f64<2, false, 3> : k_push_f64<2, false, 1>);
 }
 
 }  // namespace
 
 size_t push_smem_bytes_f64(const Ctx &c)
 {
-    return (sizeof(unsigned long long) * NCH + 48) * (size_t)c.tile_slots;
+    return f64_tile_bytes(c.tile_slots, words_f64(c)) + 48 * (size_t)c.ftile_slots;
 }
 
 int push_blocks_per_sm_f64(const Ctx &c)
 {
-    size_t bytes = push_smem_bytes_f64(c);
-    occupancy_f64<3, false>(bytes);
-    occupancy_f64<2, false>(bytes);
-    occupancy_f64<3, true>(bytes);
-    occupancy_f64<2, true>(bytes);
-    int nb = c.ndim == 3 ? occupancy_f64<3, true>(bytes) : occupancy_f64<2, true>(bytes);
+    int nb = 0;
+    for (bool full : {false, true}) {
+        auto k = kernel_f64(c, full);
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PUSH_SMEM_LIMIT);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, PUSH_THREADS, push_smem_bytes_f64(c));
+    }
     return nb < 1 ? 1 : nb;
 }
 
 int launch_push_f64(const Ctx &c, const SortScratch &s, int32_t *work_ctr, int cur_out, int full, double dt,
                     int grid_blocks, cudaStream_t st)
 {
-    size_t bytes = push_smem_bytes_f64(c);
     cudaMemsetAsync(work_ctr, 0, sizeof(int32_t), st);
-    if (c.ndim == 3) {
-        if (full)
-            k_push_f64<3, true><<<grid_blocks, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
-        else
-            k_push_f64<3, false><<<grid_blocks, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
-    } else {
-        if (full)
-            k_push_f64<2, true><<<grid_blocks, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
-        else
-            k_push_f64<2, false><<<grid_blocks, PUSH_THREADS, bytes, st>>>(c, s.items, s.nitems, work_ctr, cur_out, dt);
-    }
+    kernel_f64(c, full != 0)<<<grid_blocks, PUSH_THREADS, push_smem_bytes_f64(c), st>>>(c, s.items, s.nitems, work_ctr,
+                                                                                       cur_out, dt);
     return 1;
 }
 

@@ -663,12 +663,11 @@ int mhdpic_init(mhdpic_ctx **out, int32_t nbox, const mhdpic_grid *grids, const 
     k.ts[2] = k.tile[0] * k.tile[1];
     if (k.ndim == 3 && k.brick[0] == 4 && k.brick[1] == 4 && k.brick[2] == 4) {
         k.halves = 1;
-        // bijections of a 4x4x2 half, mod 32 for 32-bit words: x + 8 y + 68 z in
-        // 544 slots (39% less to clear and 24 KB a block more for L1 than
-        // x + 12 y + 112 z: 21.75 -> 21.46 ms for two steps of 128^3 x 32), and
-        // mod 16 within a layer for the FP64 push's 64-bit words
-        k.ts[1] = k.prec == MHDPIC_PREC_MIXED ? 8 : 12;
-        k.ts[2] = k.prec == MHDPIC_PREC_MIXED ? 68 : 112;
+        // x + 8 y + 68 z mod 32 is a bijection of a 4x4x2 half, in 544 slots
+        // (39% less to clear and 24 KB a block more for L1 than x + 12 y +
+        // 112 z: 21.75 -> 21.46 ms for two steps of 128^3 x 32)
+        k.ts[1] = 8;
+        k.ts[2] = 68;
     } else if (k.ndim == 2 && k.brick[0] == 8 && k.brick[1] == 8) {
         k.halves = 1;
         k.ts[1] = 24;    // (x + 24 y) mod 32 is a bijection of an 8x4 half

@@ -62,3 +62,25 @@ def test_fp64_push_matches_oracle(ndim, units, faces, steps):
     assert np.all(np.abs(vg - st.v) <= 1e-12 * steps * np.sqrt((st.v ** 2).sum(0)))
     assert eng.status() == 0
     eng.close()
+
+
+@pytest.mark.parametrize("one_cell", [False, True])
+@pytest.mark.parametrize("ndim,brick", [(3, (8, 8, 8)), (2, (36, 36, 1)), (2, (32, 32, 1)), (3, (4, 4, 2))])
+def test_fp64_tile_words_give_the_same_integers(ndim, brick, one_cell):
+    """Bricks too large for the 32-bit words (8^3, 36^2) take a 64-bit tile: the
+    sums are integers, the same for every brick, tile and order; with every
+    particle in one cell the words are as full as they get (2,646 particles in
+    2-D and 5,000 in 3-D, more than an item takes)."""
+    box = _box(ndim, 1.0, False)
+    if one_cell:
+        box.cell[:] = box.cell[0]
+    got = []
+    for b in ((0, 0, 0), brick):
+        eng = m.Engine([box], precision=m.MHDPIC_PREC_FP64, device="cuda:0", brick=b)
+        for _ in range(3):
+            eng.interp_push(box.dt, 1)
+        got.append([eng.deposits(i).clone() for i in (0, 1)])
+        assert eng.status() == 0
+        eng.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)

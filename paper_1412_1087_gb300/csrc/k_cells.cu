@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) k_totals_partial(Ctx c, int nchunks, int6
         for (int d = 0; d < 3; ++d)
             acc[4 + d] += m_cr * v[d];
         // E_k = v^2 / (gamma + 1)
-        acc[7] += m_cr * (v2 * reciprocal(fma(s * reciprocal_sqrt(s), invC, 1.0)));
+        acc[7] += m_cr * (v2 * reciprocal(fma(square_root(s), invC, 1.0)));
     }
     __shared__ double red[8][256];
     for (int q = 0; q < 8; ++q)

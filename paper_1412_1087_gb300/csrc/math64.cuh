@@ -52,6 +52,17 @@ __device__ __forceinline__ double reciprocal_sqrt(double s)
     return fma(y, fma(e, 0.375, 0.5) * e, y);
 }
 
+// sqrt(s) from the same estimate, one operation less than s reciprocal_sqrt(s)
+__device__ __forceinline__ double square_root(double s)
+{
+    if (!plain_range(s))
+        return sqrt(s);
+    const double y = widen(rsqrtf(cut_to_float(s)));
+    const double r = s * y;
+    const double e = fma(-r, y, 1.0);
+    return fma(r, fma(e, 0.375, 0.5) * e, r);
+}
+
 // Whole part and rest of s, |s| < 2^31: s + 1.5 2^52 rounded down holds
 // floor(s) in its low word.
 __device__ __forceinline__ void floor_split(double s, int &whole, double &rest)

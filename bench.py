@@ -62,10 +62,10 @@ GAS_CORRECT_BYTES = 32 + 56 + 56 + 56 + 32
 # one); traffic scales with the particle count (cells scale alike at fixed
 # particles per cell).  Remove an entry whenever its kernel changes, until it
 # is measured again.  Both from 'ncu --set full' of one launch: the 3-D beam at
-# 64^3 x 32 (590.9 MB for 8,388,608 particles), Bell at 512^2 x 64 (1183.5 MB
+# 64^3 x 32 (686.6 MB for 8,388,608 particles), Bell at 512^2 x 64 (1255.1 MB
 # for 16,777,216 particles); commands in profiles/.
-PUSH_TRAFFIC_BYTES_PER_PARTICLE = {"alfvenic_beam_3d": 590.871296e6 / 8388608,
-                                   "bell_2d": 1183.462144e6 / 16777216}
+PUSH_TRAFFIC_BYTES_PER_PARTICLE = {"alfvenic_beam_3d": 686.579456e6 / 8388608,
+                                   "bell_2d": 1255.07576e6 / 16777216}
 # int32 shared-memory atomic adds per particle of the push's two TSC deposits:
 # 8 channels on 3^D cells, one word per contribution for the charge density
 # and two (hi, lo) for the other seven channels, and one contribution count
@@ -77,10 +77,10 @@ SMEM_ATOMIC_CYCLES = 1.1
 # Shared-memory wavefronts per particle of the push (its shared loads,
 # stores and atomics, bank conflicts included), from the same captures as
 # the traffic above (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum:
-# 307,599,692 for the 3-D beam at 64^3 x 32, 186,552,819 for Bell at
+# 303,467,242 for the 3-D beam at 64^3 x 32, 185,621,316 for Bell at
 # 512^2 x 64); remove an entry whenever its kernel changes.
-PUSH_SHARED_WAVEFRONTS_PER_PARTICLE = {"alfvenic_beam_3d": 307599692 / 8388608,
-                                       "bell_2d": 186552819 / 16777216}
+PUSH_SHARED_WAVEFRONTS_PER_PARTICLE = {"alfvenic_beam_3d": 303467242 / 8388608,
+                                       "bell_2d": 185621316 / 16777216}
 # wavefronts per SM-cycle that a standalone probe of warp-wide shared atomic
 # adds reaches on this GPU with the deposit tile's own address pattern (the
 # highest rate measured for the pipe)
@@ -680,9 +680,10 @@ def run_native(args):
     # sort every step the feedback on a second stream beside the sort; on
     # this box in this run
     fused_form = "feedback_beside_sort" if args.sort_every == 1 else "one_launch"
+    has_form = args.sort_every == 1 or bool(eng.step_fusion())   # one-launch steps up to a size only
     fusion = {"one_launch_steps": bool(eng.step_fusion()) and args.sort_every != 1,
-              "form": fused_form if eng.step_fusion() else "separate_launches"}
-    if eng.step_fusion() and args.fusion_ab:
+              "form": fused_form if has_form else "separate_launches"}
+    if has_form and args.fusion_ab:
         ab = {}
         for fuse in (False, True):
             eng.set_step_fusion(fuse)

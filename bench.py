@@ -75,12 +75,14 @@ SMEM_ATOMICS_PER_PARTICLE = {3: 27 * (1 + 7 * 2) + 2, 2: 9 * (1 + 7 * 2) + 2}
 # banks, each adding its own value (standalone probe on a GB300)
 SMEM_ATOMIC_CYCLES = 1.1
 # Shared-memory wavefronts per particle of the push (its shared loads,
-# stores and atomics, bank conflicts included), from the same captures as
-# the traffic above (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum:
-# 303,467,242 for the 3-D beam at 64^3 x 32, 185,621,316 for Bell at
-# 512^2 x 64); remove an entry whenever its kernel changes.
-PUSH_SHARED_WAVEFRONTS_PER_PARTICLE = {"alfvenic_beam_3d": 303467242 / 8388608,
-                                       "bell_2d": 185621316 / 16777216}
+# stores and atomics, bank conflicts included;
+# l1tex__data_pipe_lsu_wavefronts_mem_shared.sum), as first captured:
+# 307,599,692 for the 3-D beam at 64^3 x 32, 186,552,819 for Bell at
+# 512^2 x 64.  The atomics are the same since; the captures in profiles/ read
+# 303,467,242 and 185,621,316 (1.3% and 0.5% less), so the fractions of the
+# pipe formed from these are that much high.
+PUSH_SHARED_WAVEFRONTS_PER_PARTICLE = {"alfvenic_beam_3d": 307599692 / 8388608,
+                                       "bell_2d": 186552819 / 16777216}
 # wavefronts per SM-cycle that a standalone probe of warp-wide shared atomic
 # adds reaches on this GPU with the deposit tile's own address pattern (the
 # highest rate measured for the pipe)
